@@ -8,6 +8,7 @@ struct PhaseP {
     int oi, rx, ry, px, py, umax;
     int a1, n1, a2, n2, M1;  // this band's anchor rows: m in [a1, a1+n1) u [a2, a2+n2)
     int ntask;
+    int att;  // attempts of the phase over the whole lattice
 };
 
 // floor(a / 2^sh) and ceil(a / 2^sh) for any sign of a (the row spacing py of an
@@ -49,6 +50,7 @@ __device__ void phase_params(int geometry, int Lx, int Ly, int W, int Y0, int Y1
     P->a2 = a2; P->n2 = max(0, b2 - a2 + 1);
     P->M1 = M1;
     P->ntask = (P->n1 + P->n2) * W;
+    P->att = Kx * My;
 }
 
 // Phase parameters of (sweep s, phase f) and the anchor rows whose row lies in
@@ -60,6 +62,7 @@ struct PhaseR {
     int oi, rx, ry, px, py, umax;
     int a[4], c[4];
     int ntask;
+    int att;  // attempts of the phase over the whole lattice
 };
 
 __device__ void phase_ranges(int geometry, int Lx, int Ly, int W, int lo, int hi, uint32_t k0,
@@ -111,6 +114,7 @@ __device__ void phase_ranges(int geometry, int Lx, int Ly, int W, int lo, int hi
     P->oi = oi; P->rx = rx; P->ry = ry; P->px = px; P->py = py;
     P->umax = px * (Kx - 1);
     P->ntask = total * W;
+    P->att = Kx * My;
 }
 
 // Bits p of the word at x0 with x0 + p in [lo, hi].
@@ -147,128 +151,113 @@ __device__ __forceinline__ void fa(uint32_t a, uint32_t b, uint32_t c, uint32_t 
     cy = (a & b) | (c & (a ^ b));
 }
 
+// Bit planes of S, the number of like neighbours an unlike pair has among the six
+// sites that only one of the two touches: like a among a's three, like b among b's
+// three (0..6).
 struct Planes {
-    uint32_t s0, s1, s2, s3;
+    uint32_t s0, s1, s2;
 };
 
-// Bit-sliced sum of ten 1-bit inputs (0..10).
-__device__ __forceinline__ Planes count10(uint32_t e0, uint32_t e1, uint32_t e2, uint32_t e3,
-                                          uint32_t e4, uint32_t e5, uint32_t e6, uint32_t e7,
-                                          uint32_t e8, uint32_t e9)
+// Planes of S for unlike pairs from the exclusive neighbours u1..u3 of a and w1..w3
+// of b.  With tb = ~ta, the count of u equal to ta is the 2-bit sum of the u, its
+// bits complemented where ta = 0 (3 - n is the complement of n), and the count of w
+// equal to tb that of the w, complemented where ta = 1; the low bit of their sum no
+// longer depends on ta.  Meaningless at positions of like pairs, which no caller reads.
+__device__ __forceinline__ Planes count_unlike(uint32_t ta, uint32_t u1, uint32_t u2, uint32_t u3, uint32_t w1,
+                                               uint32_t w2, uint32_t w3)
 {
-    uint32_t sa, ca, sb, cb, sc, cc, sd, cd;
-    fa(e0, e1, e2, sa, ca);
-    fa(e3, e4, e5, sb, cb);
-    fa(e6, e7, e8, sc, cc);
-    fa(sa, sb, sc, sd, cd);             // weight-1: sd; weight-2: cd
+    uint32_t su, cu, sw, cw;
+    fa(u1, u2, u3, su, cu);
+    fa(w1, w2, w3, sw, cw);
+    const uint32_t carry = ~(su ^ ta) & (sw ^ ta);
     Planes P;
-    P.s0 = sd ^ e9;
-    uint32_t ce = sd & e9;              // weight 2
-    uint32_t s2a, c2a, s2b, c2b;
-    fa(ca, cb, cc, s2a, c2a);           // weight 2 -> s2a (w2), c2a (w4)
-    fa(cd, ce, s2a, s2b, c2b);          // weight 2 -> s2b (w2), c2b (w4)
-    P.s1 = s2b;
-    P.s2 = c2a ^ c2b;
-    P.s3 = c2a & c2b;
+    P.s0 = ~(su ^ sw);
+    P.s1 = ~(cu ^ cw) ^ carry;
+    const uint32_t x = ~(cu ^ ta), y = cw ^ ta;
+    P.s2 = (x & y) | (carry & (x | y));
     return P;
 }
 
-// Bit-sliced sum of six 1-bit inputs (0..6).
-__device__ __forceinline__ Planes count6(uint32_t e0, uint32_t e1, uint32_t e2, uint32_t e3,
-                                         uint32_t e4, uint32_t e5)
-{
-    uint32_t sa, ca, sb, cb, s2, c2;
-    fa(e0, e1, e2, sa, ca);
-    fa(e3, e4, e5, sb, cb);
-    Planes P;
-    P.s0 = sa ^ sb;
-    fa(ca, cb, sa & sb, s2, c2);
-    P.s1 = s2;
-    P.s2 = c2;
-    P.s3 = 0u;
-    return P;
-}
-
-__device__ __forceinline__ uint32_t eqm(uint32_t v, uint32_t t) { return ~(v ^ t); }
-
-// Positions that need a draw: the exchange raises the energy when omega > 0
-// (sign > 0: S > z - 1) or lowers it when omega < 0 (sign < 0: S < z - 1).
-template <int G>
+// Positions that need a draw: the exchange changes n_unlike by 2 (S - 3), so it
+// raises the energy when omega > 0 and S > 3 (sign > 0), or omega < 0 and S < 3.
 __device__ __forceinline__ uint32_t draw_positions(const Planes &S, int sign)
 {
-    uint32_t up, down;
-    if (G == kTRI6) {  // z - 1 = 5, S in 0..10
-        up = S.s3 | (S.s2 & S.s1);                     // S >= 6
-        down = ~(S.s3 | (S.s2 & (S.s1 | S.s0)));       // S <= 4
-    } else {           // z - 1 = 3, S in 0..6
-        up = S.s2;                                     // S >= 4
-        down = ~(S.s2 | (S.s1 & S.s0));                // S <= 2
-    }
-    return sign > 0 ? up : (sign < 0 ? down : 0u);
+    return sign > 0 ? S.s2 : (sign < 0 ? ~(S.s2 | (S.s1 & S.s0)) : 0u);
+}
+
+// Entry k of the kernels' threshold table: the job's threshold of a pair with S = k.
+// The job's table counts the like neighbours of both sites; on the triangular
+// lattice an unlike pair has two common neighbours, each like exactly one of the
+// two, so its sums are S + 2.
+__device__ __forceinline__ uint64_t pair_threshold(const SweepJob &J, int k)
+{
+    return k < 7 ? J.thr[k + (J.geometry == kTRI6 ? 2 : 0)] : 0ull;
+}
+constexpr int kThrEntries = 8;
+
+// Bits of S at position p, the index into the threshold table.
+__device__ __forceinline__ uint32_t plane_bits(const Planes &S, int p)
+{
+    return ((S.s0 >> p) & 1u) | (((S.s1 >> p) & 1u) << 1) | (((S.s2 >> p) & 1u) << 2);
+}
+
+// n_unlike change / 2 of the accepted exchanges acc (na of them).
+__device__ __forceinline__ int half_dn(const Planes &S, uint32_t acc, int na)
+{
+    return __popc(S.s0 & acc) + 2 * __popc(S.s1 & acc) + 4 * __popc(S.s2 & acc) - 3 * na;
 }
 
 // Bit-sliced evaluation of the word at x0 = 32 j of the anchor row whose padded
 // shared-memory row is r0 (rows r0 - 2 RW .. r0 + 2 RW are its neighbours): the
 // types ta, tb of a = (x, y) and b = a + o for all 32 positions x0 + p, and the bit
-// planes of S = same_a + same_b.
+// planes of S.  A pair that moves is unlike, so a neighbour of both sites is like
+// exactly one of them and adds a constant: only the six neighbours of one site
+// alone are compared (10 comparisons and adders of 10 inputs before, 6 now).
 template <int G, int OI>
 __device__ __forceinline__ void evaluate(const uint32_t *r0, int RW, int j, uint32_t &ta,
                                          uint32_t &tb, Planes &S)
 {
     const uint32_t *rm = r0 - RW, *rp = r0 + RW;
-    const uint32_t a0 = r0[j], a1 = r0[j + 1], a2 = r0[j + 2];
-    const uint32_t Am = fsr(a0, a1, 31), A0 = a1, A1 = fsr(a1, a2, 1);
+    const uint32_t a0 = r0[j], a1 = r0[j + 1];
+    const uint32_t Am = fsr(a0, a1, 31);
+    ta = a1;
     if (G == kTRI6 && OI == 0) {
+        // a: (-1,0) (0,-1) (-1,1); b = (1,0): (2,0) (1,1) (2,-1); common (0,1) (1,-1)
+        const uint32_t a2 = r0[j + 2];
         const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
         const uint32_t p0 = rp[j], p1 = rp[j + 1], p2 = rp[j + 2];
-        const uint32_t M0 = m1, M1 = fsr(m1, m2, 1), M2 = fsr(m1, m2, 2);
-        const uint32_t A2 = fsr(a1, a2, 2);
-        const uint32_t Pm = fsr(p0, p1, 31), P0 = p1, P1 = fsr(p1, p2, 1);
-        ta = A0; tb = A1;
-        S = count10(eqm(Am, ta), eqm(P0, ta), eqm(M0, ta), eqm(M1, ta), eqm(Pm, ta),
-                    eqm(A2, tb), eqm(P1, tb), eqm(M1, tb), eqm(M2, tb), eqm(P0, tb));
+        tb = fsr(a1, a2, 1);
+        S = count_unlike(ta, Am, m1, fsr(p0, p1, 31), fsr(a1, a2, 2), fsr(p1, p2, 1), fsr(m1, m2, 2));
     } else if (G == kTRI6 && OI == 1) {
+        // a: (-1,0) (0,-1) (1,-1); b = (0,1): (1,1) (0,2) (-1,2); common (1,0) (-1,1)
         const uint32_t *rq = rp + RW;
         const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
-        const uint32_t p0 = rp[j], p1 = rp[j + 1], p2 = rp[j + 2];
+        const uint32_t p1 = rp[j + 1], p2 = rp[j + 2];
         const uint32_t q0 = rq[j], q1 = rq[j + 1];
-        const uint32_t M0 = m1, M1 = fsr(m1, m2, 1);
-        const uint32_t Pm = fsr(p0, p1, 31), P0 = p1, P1 = fsr(p1, p2, 1);
-        const uint32_t Qm = fsr(q0, q1, 31), Q0 = q1;
-        ta = A0; tb = P0;
-        S = count10(eqm(A1, ta), eqm(Am, ta), eqm(M0, ta), eqm(M1, ta), eqm(Pm, ta),
-                    eqm(P1, tb), eqm(Pm, tb), eqm(Q0, tb), eqm(A1, tb), eqm(Qm, tb));
+        tb = p1;
+        S = count_unlike(ta, Am, m1, fsr(m1, m2, 1), fsr(p1, p2, 1), q1, fsr(q0, q1, 31));
     } else if (G == kTRI6 && OI == 2) {
+        // a: (-1,0) (0,1) (-1,1); b = (1,-1): (2,-1) (1,-2) (2,-2); common (1,0) (0,-1)
         const uint32_t *rn = rm - RW;
         const uint32_t n1 = rn[j + 1], n2 = rn[j + 2];
         const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
         const uint32_t p0 = rp[j], p1 = rp[j + 1];
-        const uint32_t N1 = fsr(n1, n2, 1), N2 = fsr(n1, n2, 2);
-        const uint32_t M0 = m1, M1 = fsr(m1, m2, 1), M2 = fsr(m1, m2, 2);
-        const uint32_t Pm = fsr(p0, p1, 31), P0 = p1;
-        ta = A0; tb = M1;
-        S = count10(eqm(A1, ta), eqm(Am, ta), eqm(P0, ta), eqm(M0, ta), eqm(Pm, ta),
-                    eqm(M2, tb), eqm(M0, tb), eqm(A1, tb), eqm(N1, tb), eqm(N2, tb));
+        tb = fsr(m1, m2, 1);
+        S = count_unlike(ta, Am, p1, fsr(p0, p1, 31), fsr(m1, m2, 2), fsr(n1, n2, 1), fsr(n1, n2, 2));
     } else if (G == kSQ4 && OI == 0) {
+        // a: (-1,0) (0,1) (0,-1); b = (1,0): (2,0) (1,1) (1,-1)
+        const uint32_t a2 = r0[j + 2];
         const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
         const uint32_t p1 = rp[j + 1], p2 = rp[j + 2];
-        const uint32_t M0 = m1, M1 = fsr(m1, m2, 1);
-        const uint32_t A2 = fsr(a1, a2, 2);
-        const uint32_t P0 = p1, P1 = fsr(p1, p2, 1);
-        ta = A0; tb = A1;
-        S = count6(eqm(Am, ta), eqm(P0, ta), eqm(M0, ta), eqm(A2, tb), eqm(P1, tb),
-                   eqm(M1, tb));
-    } else {  // SQ4, (0,1)
+        tb = fsr(a1, a2, 1);
+        S = count_unlike(ta, Am, p1, m1, fsr(a1, a2, 2), fsr(p1, p2, 1), fsr(m1, m2, 1));
+    } else {
+        // SQ4; a: (1,0) (-1,0) (0,-1); b = (0,1): (1,1) (-1,1) (0,2)
         const uint32_t *rq = rp + RW;
-        const uint32_t m1 = rm[j + 1];
+        const uint32_t a2 = r0[j + 2];
         const uint32_t p0 = rp[j], p1 = rp[j + 1], p2 = rp[j + 2];
-        const uint32_t q1 = rq[j + 1];
-        const uint32_t M0 = m1;
-        const uint32_t Pm = fsr(p0, p1, 31), P0 = p1, P1 = fsr(p1, p2, 1);
-        const uint32_t Q0 = q1;
-        ta = A0; tb = P0;
-        S = count6(eqm(A1, ta), eqm(Am, ta), eqm(M0, ta), eqm(P1, tb), eqm(Pm, tb),
-                   eqm(Q0, tb));
+        tb = p1;
+        S = count_unlike(ta, fsr(a1, a2, 1), Am, rm[j + 1], fsr(p1, p2, 1), fsr(p0, p1, 31), rq[j + 1]);
     }
 }
 
@@ -287,12 +276,8 @@ __device__ __forceinline__ uint32_t draw_accepts(uint32_t dmask, const Planes &S
         dm &= dm - 1u;
         uint32_t r1, r2;
         philox2_w0_key(site_base + (uint32_t)p1, site_base + (uint32_t)p2, dk, r1, r2);
-        const uint32_t S1 = ((S.s0 >> p1) & 1u) | (((S.s1 >> p1) & 1u) << 1) |
-                            (((S.s2 >> p1) & 1u) << 2) | (((S.s3 >> p1) & 1u) << 3);
-        const uint32_t S2 = ((S.s0 >> p2) & 1u) | (((S.s1 >> p2) & 1u) << 1) |
-                            (((S.s2 >> p2) & 1u) << 2) | (((S.s3 >> p2) & 1u) << 3);
-        if ((uint64_t)r1 < thr[S1]) acc |= 1u << p1;
-        if ((uint64_t)r2 < thr[S2]) acc |= 1u << p2;
+        if ((uint64_t)r1 < thr[plane_bits(S, p1)]) acc |= 1u << p1;
+        if ((uint64_t)r2 < thr[plane_bits(S, p2)]) acc |= 1u << p2;
     }
     return acc;
 }
@@ -306,11 +291,12 @@ __device__ __forceinline__ uint32_t draw_accepts(uint32_t dmask, const Planes &S
 // shared atomics.  One scan and one pass serve both tasks, so a pass drains about
 // twice the draws of one task per lane.  When the warp has more than kDrawQueue2
 // draws, each lane draws its own.  Every lane of the warp must call it.  Region q
-// (16-byte aligned, kDrawQueue2Words words): planes uint4[2][32], sites
-// uint32[2][32], accept words uint32[2][32] (zero on entry and on return),
+// (16-byte aligned, kDrawQueue2Words words): records uint4[2][32] (the three planes
+// and the first site), accept words uint32[2][32] (zero on entry and on return),
 // entries uint16[kDrawQueue2].
 constexpr int kDrawQueue2 = 512;
-constexpr int kDrawQueue2Words = 2 * 32 * 4 + 2 * 32 + 2 * 32 + kDrawQueue2 / 2;
+constexpr int kDrawQueue2Acc = 2 * 32 * 4;  // word offset of the accept words
+constexpr int kDrawQueue2Words = kDrawQueue2Acc + 2 * 32 + kDrawQueue2 / 2;
 
 template <bool RK>  // RK: the round keys from rk (kernel parameter space); else from dk
 __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Planes &S0, uint32_t base0,
@@ -336,18 +322,11 @@ __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Plane
         acc1 = draw_accepts(dmask1, S1, base1, dk, thr);
         return;
     }
-    uint4 *const planes = (uint4 *)q;                  // [2][32]
-    uint32_t *const sites = (uint32_t *)(planes + 64);  // [2][32]
-    uint32_t *const wacc = sites + 64;                  // [2][32]
+    uint4 *const rec = (uint4 *)q;  // [2][32]
+    uint32_t *const wacc = q + kDrawQueue2Acc;  // [2][32]
     uint16_t *const ent = (uint16_t *)(wacc + 64);
-    if (dmask0 != 0u) {
-        planes[lane] = make_uint4(S0.s0, S0.s1, S0.s2, S0.s3);
-        sites[lane] = base0;
-    }
-    if (dmask1 != 0u) {
-        planes[32 + lane] = make_uint4(S1.s0, S1.s1, S1.s2, S1.s3);
-        sites[32 + lane] = base1;
-    }
+    if (dmask0 != 0u) rec[lane] = make_uint4(S0.s0, S0.s1, S0.s2, base0);
+    if (dmask1 != 0u) rec[32 + lane] = make_uint4(S1.s0, S1.s1, S1.s2, base1);
     int slot = incl - nd;
     uint32_t dm = dmask0;
     while (dm != 0u) {
@@ -371,24 +350,18 @@ __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Plane
             const bool two = k + 32 < total;
             const uint32_t e2 = two ? ent[k + 32] : e1;
             const uint32_t r1i = e1 >> 5, p1 = e1 & 31u, r2i = e2 >> 5, p2 = e2 & 31u;  // record = task*32 + lane
+            const uint4 a = rec[r1i], b = rec[r2i];
             uint32_t r1, r2;
-            if (RK) philox2_w0_rk(sites[r1i] + p1, sites[r2i] + p2, dk, rk, r1, r2);
-            else philox2_w0_key(sites[r1i] + p1, sites[r2i] + p2, dk, r1, r2);
-            const uint4 a = planes[r1i], b = planes[r2i];
-            const uint32_t Sa = ((a.x >> p1) & 1u) | (((a.y >> p1) & 1u) << 1) | (((a.z >> p1) & 1u) << 2) |
-                                (((a.w >> p1) & 1u) << 3);
-            const uint32_t Sb = ((b.x >> p2) & 1u) | (((b.y >> p2) & 1u) << 1) | (((b.z >> p2) & 1u) << 2) |
-                                (((b.w >> p2) & 1u) << 3);
-            if ((uint64_t)r1 < thr[Sa]) atomicOr(wacc + r1i, 1u << p1);
-            if (two && (uint64_t)r2 < thr[Sb]) atomicOr(wacc + r2i, 1u << p2);
+            if (RK) philox2_w0_rk(a.w + p1, b.w + p2, dk, rk, r1, r2);
+            else philox2_w0_key(a.w + p1, b.w + p2, dk, r1, r2);
+            if ((uint64_t)r1 < thr[plane_bits({a.x, a.y, a.z}, (int)p1)]) atomicOr(wacc + r1i, 1u << p1);
+            if (two && (uint64_t)r2 < thr[plane_bits({b.x, b.y, b.z}, (int)p2)]) atomicOr(wacc + r2i, 1u << p2);
         } else if (k < total) {
             const uint32_t e1 = ent[k];
             const uint32_t r1i = e1 >> 5, p1 = e1 & 31u;
-            const uint32_t r1 = RK ? philox_w0_rk(sites[r1i] + p1, dk, rk) : philox_w0_key(sites[r1i] + p1, dk);
-            const uint4 a = planes[r1i];
-            const uint32_t Sa = ((a.x >> p1) & 1u) | (((a.y >> p1) & 1u) << 1) | (((a.z >> p1) & 1u) << 2) |
-                                (((a.w >> p1) & 1u) << 3);
-            if ((uint64_t)r1 < thr[Sa]) atomicOr(wacc + r1i, 1u << p1);
+            const uint4 a = rec[r1i];
+            const uint32_t r1 = RK ? philox_w0_rk(a.w + p1, dk, rk) : philox_w0_key(a.w + p1, dk);
+            if ((uint64_t)r1 < thr[plane_bits({a.x, a.y, a.z}, (int)p1)]) atomicOr(wacc + r1i, 1u << p1);
         }
     }
     __syncwarp();

@@ -187,7 +187,7 @@ __device__ __forceinline__ void helical_flip(const HGeo &g, int lr, int j, unsig
 }
 
 struct HAcc {
-    uint32_t att, unl, drw, acc;
+    uint32_t unl, drw, acc;
     int32_t dn;
 };
 
@@ -210,12 +210,8 @@ __device__ __forceinline__ uint32_t helical_draws(uint32_t dmask, const Planes &
         c2 += c2 >= N ? -N : (c2 < 0 ? N : 0);
         uint32_t r1, r2;
         philox2_w0_key((uint32_t)c1, (uint32_t)c2, dk, r1, r2);
-        const uint32_t S1 = ((S.s0 >> p1) & 1u) | (((S.s1 >> p1) & 1u) << 1) | (((S.s2 >> p1) & 1u) << 2) |
-                            (((S.s3 >> p1) & 1u) << 3);
-        const uint32_t S2 = ((S.s0 >> p2) & 1u) | (((S.s1 >> p2) & 1u) << 1) | (((S.s2 >> p2) & 1u) << 2) |
-                            (((S.s3 >> p2) & 1u) << 3);
-        if ((uint64_t)r1 < thr[S1]) acc |= 1u << p1;
-        if ((uint64_t)r2 < thr[S2]) acc |= 1u << p2;
+        if ((uint64_t)r1 < thr[plane_bits(S, p1)]) acc |= 1u << p1;
+        if ((uint64_t)r2 < thr[plane_bits(S, p2)]) acc |= 1u << p2;
     }
     return acc;
 }
@@ -248,12 +244,11 @@ __device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGe
         Planes S;
         evaluate<kTRI6, OI>(lat + (size_t)lr * g.RW, g.RW, j, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
-        const uint32_t dmask = unl & draw_positions<kTRI6>(S, g.sign);
+        const uint32_t dmask = unl & draw_positions(S, g.sign);
         uint32_t acc = unl & ~dmask;
         acc |= helical_draws(dmask, S, (int)a0 + delta, (int)g.N, dk, thr);
         const bool own = (unsigned)(lr - g.D) < (unsigned)g.H;
         if (own) {
-            A.att += __popc(am);
             A.unl += __popc(unl);
             A.drw += __popc(dmask);
         }
@@ -261,9 +256,7 @@ __device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGe
         if (own) {
             const int na = __popc(acc);
             A.acc += na;
-            const int sum_s = __popc(S.s0 & acc) + 2 * __popc(S.s1 & acc) + 4 * __popc(S.s2 & acc) +
-                              8 * __popc(S.s3 & acc);
-            A.dn += 2 * (sum_s - 5 * na);
+            A.dn += 2 * half_dn(S, acc, na);
         }
         // b sites; with bdx = 1 the partner of anchor Lx-1 is position Lx, site 0 of
         // the next row of the b row.
@@ -299,7 +292,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
 {
     constexpr int kWarps = kHelicalThreads / 32;
     extern __shared__ __align__(16) uint32_t lat[];
-    __shared__ uint64_t thr[16];
+    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
     __shared__ uint2 sched[2];  // (colour, direction draw) of the current and the next iteration
     if (Cl.n_mcs <= 0) return;
@@ -328,7 +321,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
         if (y < 0) y += g.Ly;
         lat[idx] = helical_word(J, y, w);
     }
-    if (tid < 16) thr[tid] = J.thr[tid];
+    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
     // Iteration f of sweep s draws its colour and direction from one Philox block;
     // the last warp's lane 0 draws them one iteration ahead, off the tasks' path.
     const bool sched_lane = tid == kHelicalThreads - 32;
@@ -337,7 +330,9 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     hcluster_sync();  // every CTA of the cluster runs before any peer writes into it
 
     const long long n_unlike0 = (tid == 0 && g.rank == 0 && Cl.trace_every > 0) ? J.state[kNUnlike] : 0;
-    unsigned long long t_att = 0, t_unl = 0, t_drw = 0, t_acc = 0;
+    // Every iteration attempts one exchange per seven sites (7 | N), counted by one thread.
+    const unsigned long long t_att = tid == 0 && g.rank == 0 ? (unsigned long long)(g.N * Cl.n_mcs) : 0ull;
+    unsigned long long t_unl = 0, t_drw = 0, t_acc = 0;
     long long t_dn = 0;
     int jb = 0, pb = 0;  // iteration within the block; buffer of the current schedule entry
     int block = 0;
@@ -345,7 +340,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
         const long long s = Cl.sweep0 + it;
         const uint32_t s_lo = (uint32_t)(unsigned long long)s;
         const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
-        HAcc A = {0u, 0u, 0u, 0u, 0};
+        HAcc A = {0u, 0u, 0u, 0};
         for (int f = 0; f < 7; ++f) {
             const uint2 sc = sched[pb];
             const int kc = (int)sc.x;
@@ -400,7 +395,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
                 ++block;
             }
         }
-        t_att += A.att; t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
+        t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
         t_dn += A.dn;
         if (Cl.trace_every > 0 && (it + 1) % Cl.trace_every == 0) {
             const long long ws = hwarp_sum(t_dn);

@@ -35,9 +35,9 @@
 //
 // Evaluation.  One thread handles the anchors of one 32-site word of one anchor
 // row.  Neighbour comparisons of all 32 positions are bitwise operations summed by
-// a carry-save adder tree into bit planes of S = same_a + same_b (neighbours of a,
-// other than b, equal to a, plus neighbours of b, other than a, equal to b).  An
-// exchange changes the number of unlike contacts by dn = 2 (S - (z - 1)).  Unlike
+// carry-save adders into bit planes of S, the like ones among the six neighbours
+// that only one site of an unlike pair touches.  Its
+// exchange changes the number of unlike contacts by dn = 2 (S - 3).  Unlike
 // pairs whose S lies in the draw range draw a Philox number; the rest are accepted
 // outright (Metropolis acceptance min{1, exp(-omega dn / kT)}, steps a-c).  A
 // lane draws for its own anchors, two Philox evaluations interleaved at a time:
@@ -91,7 +91,7 @@ __device__ __forceinline__ void xor_at(uint32_t row, int RW, int q, uint32_t mas
 }
 
 struct Acc {
-    uint32_t att, unl, drw, acc;
+    uint32_t unl, drw, acc;
     int32_t dn;
 };
 
@@ -100,7 +100,6 @@ struct Geo {
     unsigned long long magicW;
     uint32_t k0, k1;
     int sign;            // draw when the exchange raises (+1) / lowers (-1) E; 0: never
-    int zm1;
     int C, rank, Y0, Y1;
     int prevY, prevH;    // band of CTA rank-1 (mod C)
     int nextY, nextH;    // band of CTA rank+1 (mod C)
@@ -234,7 +233,7 @@ __device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, con
     for (int t0 = threadIdx.x & ~31; t0 < nlane; t0 += THREADS) {
         const int tl = t0 + lane;
         uint32_t am = 0u, ta = 0u, tb = 0u;
-        Planes S = {0u, 0u, 0u, 0u};
+        Planes S = {0u, 0u, 0u};
         int ybase = 0, x0 = 0, lr = 0;
         if (tl < nlane) {
             const int t = tl >> ls;
@@ -267,13 +266,12 @@ __device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, con
             evaluate<G, OI>(lat + (size_t)lr * g.RW, g.RW, j, ta, tb, S);
         }
         const uint32_t unl = (ta ^ tb) & am;
-        const uint32_t dmask = unl & draw_positions<G>(S, g.sign);
+        const uint32_t dmask = unl & draw_positions(S, g.sign);
         uint32_t acc = unl & ~dmask;
 
         acc |= draw_accepts(dmask, S, (uint32_t)(ybase + x0), dk, thr);
         const bool own = !BLOCKED || (unsigned)(lr - g.D) < (unsigned)H;
         if (own) {
-            A.att += __popc(am);
             A.unl += __popc(unl);
             A.drw += __popc(dmask);
         }
@@ -281,9 +279,7 @@ __device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, con
             if (own) {
                 const int na = __popc(acc);
                 A.acc += na;
-                const int sum_s = __popc(S.s0 & acc) + 2 * __popc(S.s1 & acc) +
-                                  4 * __popc(S.s2 & acc) + 8 * __popc(S.s3 & acc);
-                A.dn += 2 * (sum_s - g.zm1 * na);
+                A.dn += 2 * half_dn(S, acc, na);
             }
             const int j = x0 >> 5;
             // b sites; with bdx = 1 the pair of anchor Lx-1 wraps to site 0.
@@ -337,7 +333,7 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
                                                const TaskTab *tt, int t, bool valid, TaskPrep &T, Acc &A)
 {
     uint32_t am = 0u, ta = 0u, tb = 0u;
-    Planes S = {0u, 0u, 0u, 0u};
+    Planes S = {0u, 0u, 0u};
     int ybase = 0, j = 0, lr = 0;
     if (valid) {
         const int mi = (int)(((unsigned long long)t * g.magicW) >> 32);
@@ -360,7 +356,7 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
         evaluate<G, OI>(lat + (size_t)lr * g.RW, g.RW, j, ta, tb, S);
     }
     const uint32_t unl = (ta ^ tb) & am;
-    T.dmask = unl & draw_positions<G>(S, g.sign);
+    T.dmask = unl & draw_positions(S, g.sign);
     T.acc = unl & ~T.dmask;
     T.S = S;
     T.base = (uint32_t)(ybase + (j << 5));
@@ -368,7 +364,6 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
     T.j = j;
     T.own = (unsigned)(lr - g.D) < (unsigned)(g.Y1 - g.Y0);
     if (T.own) {
-        A.att += __popc(am);
         A.unl += __popc(unl);
         A.drw += __popc(T.dmask);
     }
@@ -383,9 +378,7 @@ __device__ __forceinline__ void band_task_finish(const Geo &g, const TaskPrep &T
     if (T.own) {
         const int na = __popc(acc);
         A.acc += na;
-        const int sum_s = __popc(T.S.s0 & acc) + 2 * __popc(T.S.s1 & acc) + 4 * __popc(T.S.s2 & acc) +
-                          8 * __popc(T.S.s3 & acc);
-        A.dn += 2 * (sum_s - g.zm1 * na);
+        A.dn += 2 * half_dn(T.S, acc, na);
     }
     const int j = T.j, lr = T.lr, x0 = j << 5;
     unsigned long long mb = (unsigned long long)acc << bdx;
@@ -559,7 +552,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     constexpr int kWarps = THREADS / 32;
     extern __shared__ __align__(16) uint32_t lat[];
     __shared__ PhaseR pp[2][8];
-    __shared__ uint64_t thr[16];
+    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
     __shared__ uint32_t tab_am[2][kTabW];   // tables of the current and the next phase
     __shared__ int2 tab_row[2][kTabRows];
@@ -574,7 +567,6 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     Geo g;
     g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = J.RW; g.magicW = J.magicW;
     g.k0 = J.key0; g.k1 = J.key1;
-    g.zm1 = (J.geometry == kTRI6 ? 6 : 4) - 1;
     // The host's draw range is [z, 2(z-1)] (omega > 0), [0, z-2] (omega < 0) or empty.
     g.sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
     g.C = C;
@@ -606,7 +598,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         if (y < 0) y += g.Ly;
         lat[idx] = padded_word(J.lat, J.packing, J.pitch, y, w, g.Lx, g.W);
     }
-    if (tid < 16) thr[tid] = J.thr[tid];
+    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
     // The last three warps prepare the next phase while the phase runs: its anchor
     // masks, its rows, and (lane 0) one schedule entry of the next sweep.
     const int warp = tid >> 5;
@@ -638,7 +630,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         const uint32_t s_lo = (uint32_t)(unsigned long long)s;
         const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
         const int buf = (int)(it & 1);
-        Acc A = {0u, 0u, 0u, 0u, 0};
+        Acc A = {0u, 0u, 0u, 0};
         for (int f = 0; f < 8; ++f) {
             const bool last = f == 7 && it + 1 == Cl.n_mcs;
             if ((table_warp || row_warp) && !last) {
@@ -656,8 +648,10 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
             // Phase f of the next sweep: one schedule entry per phase.  (Entry f of the
             // other buffer was last read in phase f of the previous sweep; phase 0's is
             // written here before phase 7 builds its task table from it.)
-            if (sched_warp && (tid & 31) == 0 && it + 1 < Cl.n_mcs)
-                phase_table(J, g, K, s + 1, f, &pp[buf ^ 1][f]);
+            if (sched_warp && (tid & 31) == 0) {
+                if (it + 1 < Cl.n_mcs) phase_table(J, g, K, s + 1, f, &pp[buf ^ 1][f]);
+                if (rank == 0) t_att += (unsigned long long)pp[buf][f].att;  // the lattice's, counted once
+            }
             const PhaseR P = pp[buf][f];
             const TaskTab Tc = {tab_am[f & 1], tab_row[f & 1], kTabW, kTabRows};
             const TaskTab *tt = &Tc;
@@ -679,7 +673,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
                 phase_barrier(C);
             }
         }
-        t_att += A.att; t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
+        t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
         t_dn += A.dn;
         // Energy trace: each CTA adds its cumulative dn; CTA 0 adds the start value
         // (the launcher zeroes the trace buffer).
@@ -788,7 +782,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     constexpr int kWarps = THREADS / 32;
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ PhaseR pp[8];
-    __shared__ uint64_t thr[16];
+    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
     __shared__ __align__(8) unsigned long long copy_bar;
     // The next launch may be scheduled now; it waits for this one before it reads.
@@ -797,7 +791,6 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     Geo g;
     g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = band_row_words(J.W); g.magicW = J.magicW;
     g.k0 = J.key0; g.k1 = J.key1;
-    g.zm1 = (J.geometry == kTRI6 ? 6 : 4) - 1;
     g.sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
     g.C = (int)gridDim.x;
     g.rank = (int)blockIdx.x;
@@ -823,7 +816,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     }
     // Everything below reads what earlier launches on the stream wrote.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid < 16) thr[tid] = J.thr[tid];
+    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
     const long long s = J.state[kSweepBase] + k;
     const uint32_t s_lo = (uint32_t)(unsigned long long)s;
     const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
@@ -903,11 +896,11 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
         __syncthreads();
     }
 
-    Acc A = {0u, 0u, 0u, 0u, 0};
+    Acc A = {0u, 0u, 0u, 0};
     // the warps' draw queues follow the rows (H + 2D rows of the tallest band)
     uint32_t *const dq = smem + (size_t)(H + 2 * g.D) * RWb + (size_t)(tid >> 5) * kDrawQueue2Words;
-    dq[2 * 32 * 4 + 2 * 32 + (tid & 31)] = 0u;       // the queue's accept words start at zero
-    dq[2 * 32 * 4 + 2 * 32 + 32 + (tid & 31)] = 0u;
+    dq[kDrawQueue2Acc + (tid & 31)] = 0u;  // the queue's accept words start at zero
+    dq[kDrawQueue2Acc + 32 + (tid & 31)] = 0u;
     for (int j = 0; j < K; ++j) {
         const PhaseR P = pp[j];
         uint32_t *const t = tab_base + (size_t)j * (tab_w + 2 * tab_rows);
@@ -957,7 +950,10 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
         }
     }
 
-    long long vals[5] = {(long long)A.att, (long long)A.unl, (long long)A.drw, (long long)A.acc,
+    long long att = 0;
+    if (blockIdx.x == 0 && tid == 0)
+        for (int j = 0; j < K; ++j) att += pp[j].att;  // the whole lattice's, counted once
+    long long vals[5] = {att, (long long)A.unl, (long long)A.drw, (long long)A.acc,
                          (long long)A.dn};
 #pragma unroll
     for (int q = 0; q < 5; ++q) {

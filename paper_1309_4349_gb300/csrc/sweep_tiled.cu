@@ -26,7 +26,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
 struct Acc {
-    uint32_t att, unl, drw, acc;
+    uint32_t unl, drw, acc;
     int32_t dn;
 };
 
@@ -52,7 +52,7 @@ __device__ __forceinline__ void flip_store(const SweepJob &J, int y, int j, unsi
 
 template <int G, int OI>
 __device__ __forceinline__ void run_tiles(const uint32_t *tile, const SweepJob &J, const PhaseP &P,
-                                          int Y0, int sign, int zm1, const uint64_t *thr, int f,
+                                          int Y0, int sign, const uint64_t *thr, int f,
                                           uint32_t s_lo, uint32_t s_hi, Acc &A)
 {
     constexpr int bdy = OI == 0 ? 0 : (OI == 1 ? 1 : -1);
@@ -71,18 +71,15 @@ __device__ __forceinline__ void run_tiles(const uint32_t *tile, const SweepJob &
         Planes S;
         evaluate<G, OI>(tile + (size_t)(y - Y0 + 2) * J.RW, J.RW, j, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
-        const uint32_t dmask = unl & draw_positions<G>(S, sign);
+        const uint32_t dmask = unl & draw_positions(S, sign);
         uint32_t acc = unl & ~dmask;
         acc |= draw_accepts(dmask, S, (uint32_t)(y * J.Lx + x0), dk, thr);
-        A.att += __popc(am);
         A.unl += __popc(unl);
         A.drw += __popc(dmask);
         if (acc) {
             const int na = __popc(acc);
             A.acc += na;
-            const int sum_s = __popc(S.s0 & acc) + 2 * __popc(S.s1 & acc) +
-                              4 * __popc(S.s2 & acc) + 8 * __popc(S.s3 & acc);
-            A.dn += 2 * (sum_s - zm1 * na);
+            A.dn += 2 * half_dn(S, acc, na);
             unsigned long long mb = (unsigned long long)acc << bdx;
             bool wrap0 = false;  // the pair of anchor Lx-1 wraps to site 0
             if (bdx == 1) {
@@ -119,7 +116,7 @@ tiled_phase_kernel(const SweepJob J, int H, int k, int f)
 {
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ PhaseP P;
-    __shared__ uint64_t thr[16];
+    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
 
     const int tid = threadIdx.x;
@@ -135,24 +132,24 @@ tiled_phase_kernel(const SweepJob J, int H, int k, int f)
         tile[idx] = padded_word(J.lat, J.packing, J.pitch, y, w, J.Lx, J.W);
     }
     if (tid == 0) phase_params(J.geometry, J.Lx, J.Ly, J.W, Y0, Y1, J.key0, J.key1, s, f, &P);
-    if (tid < 16) thr[tid] = J.thr[tid];
+    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
     __syncthreads();
 
-    const int zm1 = (J.geometry == kTRI6 ? 6 : 4) - 1;
     const int sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
     const uint32_t s_lo = (uint32_t)(unsigned long long)s;
     const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
-    Acc A = {0u, 0u, 0u, 0u, 0};
+    Acc A = {0u, 0u, 0u, 0};
     if (J.geometry == kTRI6) {
-        if (P.oi == 0) run_tiles<kTRI6, 0>(tile, J, P, Y0, sign, zm1, thr, f, s_lo, s_hi, A);
-        else if (P.oi == 1) run_tiles<kTRI6, 1>(tile, J, P, Y0, sign, zm1, thr, f, s_lo, s_hi, A);
-        else run_tiles<kTRI6, 2>(tile, J, P, Y0, sign, zm1, thr, f, s_lo, s_hi, A);
+        if (P.oi == 0) run_tiles<kTRI6, 0>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
+        else if (P.oi == 1) run_tiles<kTRI6, 1>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
+        else run_tiles<kTRI6, 2>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
     } else {
-        if (P.oi == 0) run_tiles<kSQ4, 0>(tile, J, P, Y0, sign, zm1, thr, f, s_lo, s_hi, A);
-        else run_tiles<kSQ4, 1>(tile, J, P, Y0, sign, zm1, thr, f, s_lo, s_hi, A);
+        if (P.oi == 0) run_tiles<kSQ4, 0>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
+        else run_tiles<kSQ4, 1>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
     }
 
-    long long vals[5] = {(long long)A.att, (long long)A.unl, (long long)A.drw, (long long)A.acc,
+    const long long att = blockIdx.x == 0 && tid == 0 ? P.att : 0;  // the whole phase's, counted once
+    long long vals[5] = {att, (long long)A.unl, (long long)A.drw, (long long)A.acc,
                          (long long)A.dn};
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
