@@ -142,9 +142,10 @@ klmc_status klmc_sweep_traced(klmc_ctx *c, int64_t n_mcs, int64_t trace_every,
 
 /* Number of unlike contacts (kept exactly, updated by every accepted exchange)
  * and E/kT = omega/kT * n_unlike (energy model of the omega_AB equation).
- * Synchronises.  Either pointer may be NULL.  KLMC_ETIMEOUT if a tiled launch
- * of this handle gave up its bounded wait for its row copies: that launch left
- * its band unwritten, so the lattice is no longer a state of the chain. */
+ * Synchronises.  Either pointer may be NULL.  KLMC_ETIMEOUT if a launch
+ * of this handle gave up a bounded wait for its row copies (the tiled path, whose
+ * launch then leaves its band unwritten, or a cluster's exchange): the lattice is no
+ * longer a state of the chain. */
 klmc_status klmc_energy(klmc_ctx *c, int64_t *n_unlike, double *energy_over_kT);
 
 /* Recounts n_unlike from the lattice on the device (every bond once) without
@@ -339,9 +340,10 @@ klmc_status klmc_destroy(klmc_ctx *c);
  * advanced together by the resident kernel, one thread-block cluster per replica.
  * Each call chooses the launch shapes of the replicas it advances: a replica with
  * a fixed shape (params.cluster or params.threads set) keeps it; replicas with
- * automatic shapes keep theirs (tuned, else automatic) while the call's CTAs fit
- * the GPU's SMs, and otherwise run at half the CTAs per replica (where the band
- * still fits shared memory) with 128 threads per CTA, so that several CTAs share
+ * automatic shapes keep theirs (tuned, else automatic), or that of bands of at least
+ * 24 rows, while the call's CTAs fit the GPU's SMs, and otherwise run at fewer CTAs
+ * per replica (bands of at least 48 rows while those run at once, else 64) with 128
+ * threads per CTA, so that several CTAs share
  * an SM.  Replicas of one shape form one launch, larger lattices first; the
  * launches of different shapes run on internal streams forked from and joined
  * back to the stream of reps[0], which every replica uses.  The trajectory of a

@@ -162,17 +162,22 @@ klmc_status validate(const klmc_params *p)
     return KLMC_OK;
 }
 
-// Automatic cluster size: the smallest power of two whose bands fit in shared
-// memory, raised while every band keeps >= 24 rows (more CTAs shorten each phase;
-// too-thin bands spend their time on halos and barriers).
-int auto_cluster(int Lx, int Ly)
+// Cluster size: the smallest power of two whose bands fit in shared memory, raised
+// while every band keeps >= min_rows rows.
+int cluster_for_rows(int Lx, int Ly, int min_rows)
 {
     const int cmax = resident_max_cluster(Ly);
     int c = 1;
     while (c < cmax && resident_smem_bytes(Lx, Ly, c) > (size_t)resident_max_smem_bytes()) c *= 2;
-    while (c * 2 <= cmax && Ly / (c * 2) >= 24) c *= 2;
+    while (c * 2 <= cmax && Ly / (c * 2) >= min_rows) c *= 2;
     return c;
 }
+
+// Automatic cluster size: bands of at least 16 rows.  More CTAs shorten each phase
+// (GB300, us per phase with half as many CTAs and with these: 64^2 0.82 / 0.76, 128^2
+// 0.93 / 0.85, 256^2 1.06 / 0.96, 300^2 1.18 / 1.04).
+constexpr int kLatencyRows = 16;
+int auto_cluster(int Lx, int Ly) { return cluster_for_rows(Lx, Ly, kLatencyRows); }
 
 // Acceptance table (Metropolis step c with u = r / 2^32): a pair whose
 // neighbour-agreement sum is S changes n_unlike by dn = 2 (S - (z - 1)); it is
@@ -201,6 +206,14 @@ klmc_status build_thresholds(double bw, int geometry, SweepJob *J)
     }
     J->draw_lo = lo;
     J->draw_hi = hi;
+    // Unlike pairs with a draw have S - (z - 1) in 1..3 (omega > 0) or -3..-1 (omega < 0):
+    // the two like-neighbour counts differ by a constant, and an unlike pair's reach no further.
+    J->draw_never = 0;
+    for (int c = 0; c < 3; ++c) {
+        const uint64_t t = hi < lo ? 0 : J->thr[bw > 0.0 ? zm1 + 1 + c : zm1 - 3 + c];
+        J->draw_t[c] = (uint32_t)(t - 1);
+        if (t == 0) J->draw_never |= 1u << c;
+    }
     return KLMC_OK;
 }
 
@@ -231,6 +244,11 @@ klmc_status ensure_clusters(klmc_ctx *c)
 
 bool tuned_shape(int Lx, int Ly, int geometry, int packing, int *cluster, int *threads, int *tuned_packing);
 
+// Bands of the shapes that fill the GPU with more lattices than run at once (GB300, 128
+// threads: 256 replicas of side 100..1024 take 169 / 150 / 163 / 207 us per step with at
+// least 48 / 64 / 80 / 100 rows).
+constexpr int kThroughputRows = 64;
+
 // Lattices of at least this many sites run faster on the tiled path, whose bands
 // use every SM, than in one cluster's shared memory (GB300, 200 MCS of square TRI6
 // lattices: 724^2 5.7 vs 4.8 ms resident, 1024^2 5.8 vs 7.1 ms, 2048^2 6.8 vs
@@ -260,7 +278,7 @@ klmc_status create_one(klmc_ctx **out, const klmc_params *p, klmc_batch *owner, 
     if (c->helical) {
         // Resident in a cluster's shared memory when the bands are tall enough for
         // blocks of iterations; otherwise one launch per iteration over the store.
-        c->cluster = p->cluster != 0 ? p->cluster : auto_cluster(p->Lx, p->Ly);
+        c->cluster = p->cluster != 0 ? p->cluster : cluster_for_rows(p->Lx, p->Ly, 24);
         if (c->cluster > 0 && helical_resident_block(p->Lx, p->Ly, c->cluster) < 2) c->cluster = -1;
         c->threads = c->cluster > 0 ? 512 : 256;
         c->auto_shape = false;
@@ -276,7 +294,7 @@ klmc_status create_one(klmc_ctx **out, const klmc_params *p, klmc_batch *owner, 
                 tiled_plan(p->Lx, p->Ly, sms).K >= 2)
                 c->cluster = -1;  // automatic choice, large: bands over every SM
         }
-        c->threads = resident_default_threads(c->cluster);
+        c->threads = resident_default_threads(p->Lx, p->Ly, c->cluster);
         int tuned_packing = c->p.packing;
         if (p->cluster == 0 && p->threads == 0 &&
             tuned_shape(p->Lx, p->Ly, p->geometry, c->auto_packing ? KLMC_PACK_AUTO : c->p.packing, &c->cluster,
@@ -469,7 +487,7 @@ klmc_status sweep_one(klmc_ctx *c, int64_t n_mcs, int64_t trace_every, int64_t *
     call.trace = (long long *)dev_trace;
     call.trace_every = trace_every;
     KLMC_CUDA(launch_resident_sweep_one(c->job, call, c->cluster, c->threads,
-                                        resident_smem_bytes(c->p.Lx, c->p.Ly, c->cluster),
+                                        resident_launch_bytes(c->p.Lx, c->p.Ly, c->cluster),
                                         c->stream));
     c->sweep += n_mcs;
     return KLMC_OK;
@@ -581,7 +599,7 @@ klmc_status probe_shape(klmc_ctx *c, const ProbeStore &ps, void *scratch_lat, lo
             call.trace = nullptr;
             call.trace_every = 0;
             KLMC_CUDA(launch_resident_sweep_one(J, call, cluster, threads,
-                                                resident_smem_bytes(c->p.Lx, c->p.Ly, cluster),
+                                                resident_launch_bytes(c->p.Lx, c->p.Ly, cluster),
                                                 c->stream));
         }
         KLMC_CUDA(cudaEventRecord(e1, c->stream));
@@ -717,12 +735,34 @@ void klmc::host::choose_shapes(const std::vector<klmc_ctx *> &cs, const std::vec
 {
     const size_t n = cs.size();
     shapes->resize(n);
-    long long ctas = 0;
-    for (size_t i = 0; i < n; ++i) {
-        (*shapes)[i] = {cs[i]->cluster, cs[i]->threads};
-        ctas += cs[i]->cluster > 0 ? cs[i]->cluster : 1;
-    }
-    if (ctas <= sm_count) return;
+    // Shapes at one level: every lattice's own, or, for automatic ones, at most as many
+    // CTAs as leave min_rows rows per band.
+    auto level = [&](int min_rows, int threads) {
+        long long ctas = 0, widest = 0;
+        for (size_t i = 0; i < n; ++i) {
+            const klmc_ctx *c = cs[i];
+            std::pair<int, int> sh{c->cluster, c->threads};
+            if (min_rows > 0 && c->auto_shape && c->cluster > 0) {
+                const int C = std::min(c->cluster, cluster_for_rows(c->p.Lx, c->p.Ly, min_rows));
+                if (threads > 0) sh = {C, threads};
+                else if (C != c->cluster) sh = {C, resident_default_threads(c->p.Lx, c->p.Ly, C)};
+            }
+            (*shapes)[i] = sh;
+            ctas += sh.first > 0 ? sh.first : 1;
+            widest += sh.first == 16;
+        }
+        // (a cluster lies within one GPC: 152 SMs hold 8 clusters of 16 CTAs, one per SM)
+        return std::max(ctas, widest * 19);
+    };
+    // One CTA per SM, else one CTA per SM with bands of at least 24 rows.
+    if (level(0, 0) <= sm_count) return;
+    if (level(24, 0) <= sm_count) return;
+    // More lattices than that: 128 threads per CTA, four CTAs per SM, as many CTAs as
+    // run at once, else bands of at least kThroughputRows rows.
+    if (level(48, 128) > 4ll * sm_count) level(kThroughputRows, 128);
+    if (!keep_longest) return;
+    // The lattices whose remaining work takes longest keep their own shapes while those
+    // CTAs fit the SMs.
     std::vector<double> work(n);
     std::vector<size_t> order(n);
     for (size_t i = 0; i < n; ++i) {
@@ -730,18 +770,12 @@ void klmc::host::choose_shapes(const std::vector<klmc_ctx *> &cs, const std::vec
         order[i] = i;
     }
     std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return work[a] > work[b]; });
-    long long left = keep_longest ? sm_count : 0;
+    long long left = sm_count;
     for (size_t i : order) {
-        klmc_ctx *c = cs[i];
-        const int own = c->cluster > 0 ? c->cluster : 1;
-        if (own <= left || !c->auto_shape || c->cluster < 1) {
-            if (own <= left) left -= own;
-            continue;
-        }
-        int half = c->cluster > 1 ? c->cluster / 2 : 1;
-        if (resident_smem_bytes(c->p.Lx, c->p.Ly, half) > (size_t)resident_max_smem_bytes())
-            half = c->cluster;
-        (*shapes)[i] = {half, 128};
+        const int own = cs[i]->cluster > 0 ? cs[i]->cluster : 1;
+        if (own > left) continue;
+        left -= own;
+        (*shapes)[i] = {cs[i]->cluster, cs[i]->threads};
     }
 }
 
@@ -814,7 +848,7 @@ klmc_status klmc_energy(klmc_ctx *c, int64_t *n_unlike, double *energy_over_kT)
     long long v[kStateSlots];
     KLMC_CUDA(cudaMemcpyAsync(v, c->state, sizeof(v), cudaMemcpyDeviceToHost, c->stream));
     KLMC_CUDA(cudaStreamSynchronize(c->stream));
-    if (v[kFault]) return fail(KLMC_ETIMEOUT, "a tiled sweep launch gave up waiting for its row copies");
+    if (v[kFault]) return fail(KLMC_ETIMEOUT, "a sweep launch gave up waiting for its row copies");
     if (n_unlike) *n_unlike = v[kNUnlike];
     if (energy_over_kT) *energy_over_kT = c->p.omega_over_kT * (double)v[kNUnlike];
     return KLMC_OK;
@@ -993,7 +1027,7 @@ klmc_status klmc_get_counters(klmc_ctx *c, klmc_counters *out)
     long long v[kStateSlots];
     KLMC_CUDA(cudaMemcpyAsync(v, c->state, sizeof(v), cudaMemcpyDeviceToHost, c->stream));
     KLMC_CUDA(cudaStreamSynchronize(c->stream));
-    if (v[kFault]) return fail(KLMC_ETIMEOUT, "a tiled sweep launch gave up waiting for its row copies");
+    if (v[kFault]) return fail(KLMC_ETIMEOUT, "a sweep launch gave up waiting for its row copies");
     out->sweeps = c->sweep;
     out->attempts = v[kAttempts];
     out->unlike = v[kUnlike];
@@ -1292,7 +1326,7 @@ klmc_status klmc_batch_sweep(klmc_batch *b, const int64_t *n_mcs)
         for (int i : g.second) {
             klmc_status st = check_resident(b->reps[i], g.first.first);
             if (st != KLMC_OK) return st;
-            const size_t sm = resident_smem_bytes(b->reps[i]->p.Lx, b->reps[i]->p.Ly, g.first.first);
+            const size_t sm = resident_launch_bytes(b->reps[i]->p.Lx, b->reps[i]->p.Ly, g.first.first);
             if (sm > smem) smem = sm;
         }
         KLMC_CUDA(cudaStreamWaitEvent(it->second.first, b->fork, 0));

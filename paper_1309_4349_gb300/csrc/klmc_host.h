@@ -85,12 +85,11 @@ inline double model_mcs_us(int Lx, int Ly, int cluster, int threads)
 
 // Launch shapes (cluster, threads) for one launch over several resident lattices,
 // lattice i to advance by steps[i].  Lattices with fixed shapes keep them.  While
-// the CTAs of all lattices at their own shapes fit the SMs, every lattice keeps its
-// own (latency) shape.  Otherwise lattices with automatic shapes run with half as
-// many CTAs (when the band still fits shared memory) and 128 threads per CTA, so
-// that several CTAs share an SM: all of them when throughput is the goal (a batch
-// call), or all but those whose remaining work takes longest, which keep their own
-// shapes as long as their CTAs fit the SMs, when latency is (a server round).
+// their CTAs run at once, one per SM, lattices with automatic shapes keep their own
+// (latency) shape, or one of higher bands.  Otherwise they run with fewer CTAs of
+// 128 threads, so that several CTAs share an SM: all of them when throughput is the
+// goal (a batch call), or all but those whose remaining work takes longest, which keep
+// their own shapes as long as their CTAs fit the SMs, when latency is (a server round).
 void choose_shapes(const std::vector<klmc_ctx *> &cs, const std::vector<int64_t> &steps,
                    int sm_count, bool keep_longest, std::vector<std::pair<int, int>> *shapes);
 

@@ -25,7 +25,7 @@ enum StateSlot : int {
     kTracePos = 8,  // next entry of the energy trace (tiled path)
     kTracePtr = 9,  // device address of the energy trace (tiled path)
     kFfn = 10,      // random-neighbour count of klmc_ffn; with slot 11, klmc_image_ffn's counts
-    kFault = 12,    // nonzero: a tiled launch gave up waiting for its row copies (band left unwritten)
+    kFault = 12,    // nonzero: a launch gave up waiting for its row copies (tiled path, cluster exchange)
     kStateSlots = 13
 };
 
@@ -45,6 +45,10 @@ struct SweepJob {
     int32_t copy_shortfall;  // test hook (0 in use): a band launch issues no row copy and waits for
                              // this many bytes instead, which nothing delivers, so its bounded wait runs out
     uint64_t thr[16];     // accept iff draw < thr[S] (S = same_a + same_b)
+    // The same table as the kernels read it: a draw r of a pair of class c (the two low bits
+    // of its S, see sweep_common.cuh) is accepted iff r <= draw_t[c], or never when bit c
+    // of draw_never is set (a threshold of 0).
+    uint32_t draw_t[3], draw_never;
     long long *state;     // StateSlot array
     uint32_t rk[2][8];    // Philox round keys of rounds 2..9: key0 + r W0, key1 + r W1
 };
@@ -61,11 +65,13 @@ struct SweepCall {
 // the per-CTA limit, and the largest cluster whose bands keep >= 4 rows.
 size_t resident_smem_bytes(int Lx, int Ly, int cluster);
 int resident_max_smem_bytes();
+// What a launch asks for: the same plus the kernel's task tables where both fit.
+size_t resident_launch_bytes(int Lx, int Ly, int cluster);
 // Phases between halo exchanges of a lattice split over `cluster` CTAs (1: a
 // cluster barrier after every phase).
 int resident_block_phases(int Lx, int Ly, int cluster);
 int resident_max_cluster(int Ly);
-int resident_default_threads(int cluster);  // 512 for one CTA, else 256
+int resident_default_threads(int Lx, int Ly, int cluster);  // 256 or 512
 
 // Batched launch: one cluster of `cluster` CTAs per job, tables in device memory;
 // launched job i is d_jobs[d_map[i]] (d_map null: job i).  The trace buffers of

@@ -317,7 +317,7 @@ klmc_status run_round(klmc_server *s)
         }
         size_t smem = 0;
         for (int i : g.second) {
-            const size_t b = klmc::resident_smem_bytes(s->active[i]->ctx->p.Lx, s->active[i]->ctx->p.Ly,
+            const size_t b = klmc::resident_launch_bytes(s->active[i]->ctx->p.Lx, s->active[i]->ctx->p.Ly,
                                                        g.first.first);
             if (b > smem) smem = b;
         }

@@ -185,20 +185,38 @@ __device__ __forceinline__ uint32_t draw_positions(const Planes &S, int sign)
     return sign > 0 ? S.s2 : (sign < 0 ? ~(S.s2 | (S.s1 & S.s0)) : 0u);
 }
 
-// Entry k of the kernels' threshold table: the job's threshold of a pair with S = k.
-// The job's table counts the like neighbours of both sites; on the triangular
-// lattice an unlike pair has two common neighbours, each like exactly one of the
-// two, so its sums are S + 2.
-__device__ __forceinline__ uint64_t pair_threshold(const SweepJob &J, int k)
-{
-    return k < 7 ? J.thr[k + (J.geometry == kTRI6 ? 2 : 0)] : 0ull;
-}
-constexpr int kThrEntries = 8;
+// Acceptance of draws.  A pair with a draw has S in 4..6 (omega > 0) or 0..2
+// (omega < 0), so the two low bits of S name its threshold: three registers and two
+// selects per draw.  Classes whose threshold is 0 never accept (DrawThr::never).
+struct DrawThr {
+    uint32_t t[3];
+    uint32_t never;
+};
 
-// Bits of S at position p, the index into the threshold table.
-__device__ __forceinline__ uint32_t plane_bits(const Planes &S, int p)
+__device__ __forceinline__ DrawThr draw_thresholds(const SweepJob &J)
 {
-    return ((S.s0 >> p) & 1u) | (((S.s1 >> p) & 1u) << 1) | (((S.s2 >> p) & 1u) << 2);
+    return {{J.draw_t[0], J.draw_t[1], J.draw_t[2]}, J.draw_never};
+}
+
+// Positions whose class never accepts.  Computed beside the draws and applied to their
+// results: a branch around this rare case, or a mask before the draws, lengthened every phase.
+__device__ __forceinline__ uint32_t never_accepted(uint32_t s0, uint32_t s1, uint32_t never)
+{
+    return (~(s0 | s1) & (0u - (never & 1u))) | (s0 & (0u - ((never >> 1) & 1u))) | (s1 & (0u - (never >> 2)));
+}
+
+// Whether draw r accepts the pair at the single bit b.
+__device__ __forceinline__ bool accepts(uint32_t r, uint32_t s0, uint32_t s1, uint32_t b, const uint32_t (&t)[3])
+{
+    const uint32_t t01 = (s0 & b) != 0u ? t[1] : t[0];
+    return r <= ((s1 & b) != 0u ? t[2] : t01);
+}
+
+__device__ __forceinline__ int bit_index(uint32_t b)  // of the highest bit; -1 for 0
+{
+    int p;
+    asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(b));
+    return p;
 }
 
 // n_unlike change / 2 of the accepted exchanges acc (na of them).
@@ -207,79 +225,130 @@ __device__ __forceinline__ int half_dn(const Planes &S, uint32_t acc, int na)
     return __popc(S.s0 & acc) + 2 * __popc(S.s1 & acc) + 4 * __popc(S.s2 & acc) - 3 * na;
 }
 
-// Bit-sliced evaluation of the word at x0 = 32 j of the anchor row whose padded
-// shared-memory row is r0 (rows r0 - 2 RW .. r0 + 2 RW are its neighbours): the
-// types ta, tb of a = (x, y) and b = a + o for all 32 positions x0 + p, and the bit
-// planes of S.  A pair that moves is unlike, so a neighbour of both sites is like
-// exactly one of them and adds a constant: only the six neighbours of one site
-// alone are compared (10 comparisons and adders of 10 inputs before, 6 now).
-template <int G, int OI>
-__device__ __forceinline__ void evaluate(const uint32_t *r0, int RW, int j, uint32_t &ta,
-                                         uint32_t &tb, Planes &S)
+// Where the neighbours of a 32-site word lie.  A shared-memory row is W words of
+// sites, the bits of its last word past the row's end zero.  l, r: distance in words
+// to the word on its left and right -- around the row's ends those of the same row
+// (periodic), or the last one of the row before and the first one of the row after
+// (helical).  top: the bit of the left word's last site; end: the bit of the word's
+// own last site.  (Rows with copies of their end sites on either side need no such
+// distances, but every flip near an end then mends copies: that took 0.15-0.21 us of a
+// 1.0-1.4 us phase of a 64^2 or 400^2 lattice on a cluster.)
+struct WordEnds {
+    int l, r;
+    int top, end;
+    bool fix;  // a last word of one site (Lx mod 32 = 1): this word is it or the one before,
+    int fix2;  // which is then followed by the word at this distance
+};
+
+// nlast: sites of a row's last word; hrow: 0 (periodic) or the row stride (helical).
+__device__ __forceinline__ WordEnds word_ends(int j, int W, int nlast, int hrow)
 {
-    const uint32_t *rm = r0 - RW, *rp = r0 + RW;
-    const uint32_t a0 = r0[j], a1 = r0[j + 1];
-    const uint32_t Am = fsr(a0, a1, 31);
-    ta = a1;
+    const bool first = j == 0, last = j == W - 1;
+    WordEnds E;
+    E.l = first ? W - 1 - hrow : -1;
+    E.r = last ? 1 - W + hrow : 1;
+    E.top = first ? nlast - 1 : 31;
+    E.end = last ? nlast - 1 : 31;
+    E.fix = nlast == 1 && j >= W - 2;
+    E.fix2 = 2 - W + hrow;
+    return E;
+}
+
+// The sites at distance -1, +1 and +2 of the word at p (32 at a time).
+__device__ __forceinline__ uint32_t window_m1(const uint32_t *p, const WordEnds &E)
+{
+    return p[0] + p[0] + (p[E.l] >> E.top);  // bits above the left word's last site are zero
+}
+__device__ __forceinline__ uint32_t window_p1(const uint32_t *p, const WordEnds &E)
+{
+    return (p[0] >> 1) + p[E.r] * (1u << E.end);
+}
+template <bool FIX>
+__device__ __forceinline__ uint32_t window_p2(const uint32_t *p, const WordEnds &E)
+{
+    const uint32_t r = p[E.r];
+    uint32_t v = (p[0] >> 2) + r * ((1u << E.end) >> 1);
+    // the sum's bits past the row's end carry nothing into it; with a last word of one
+    // site, that word's site and the last one before it look two words on
+    if (FIX && E.fix) v = E.end == 0 ? r >> 1 : (v & 0x7FFFFFFFu) | (p[E.fix2] << 31);
+    return v;
+}
+
+// Bit-sliced evaluation of the word at p of an anchor row in shared memory (rows of
+// stride RW): the types ta, tb of a = (x, y) and b = a + o for its 32 positions, and
+// the bit planes of S.  A pair that moves is unlike, so a neighbour of both sites is
+// like exactly one of them and adds a constant: only the six neighbours of one site
+// alone are compared (10 comparisons and adders of 10 inputs before, 6 now).
+// FIX: rows may have a last word of one site.
+template <int G, int OI, bool FIX>
+__device__ __forceinline__ void evaluate(const uint32_t *p, int RW, const WordEnds &E, uint32_t &ta, uint32_t &tb,
+                                         Planes &S)
+{
+    const uint32_t *pm = p - RW, *pp = p + RW;
+    ta = p[0];
+    const uint32_t Am = window_m1(p, E);
     if (G == kTRI6 && OI == 0) {
         // a: (-1,0) (0,-1) (-1,1); b = (1,0): (2,0) (1,1) (2,-1); common (0,1) (1,-1)
-        const uint32_t a2 = r0[j + 2];
-        const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
-        const uint32_t p0 = rp[j], p1 = rp[j + 1], p2 = rp[j + 2];
-        tb = fsr(a1, a2, 1);
-        S = count_unlike(ta, Am, m1, fsr(p0, p1, 31), fsr(a1, a2, 2), fsr(p1, p2, 1), fsr(m1, m2, 2));
+        tb = window_p1(p, E);
+        S = count_unlike(ta, Am, pm[0], window_m1(pp, E), window_p2<FIX>(p, E), window_p1(pp, E), window_p2<FIX>(pm, E));
     } else if (G == kTRI6 && OI == 1) {
         // a: (-1,0) (0,-1) (1,-1); b = (0,1): (1,1) (0,2) (-1,2); common (1,0) (-1,1)
-        const uint32_t *rq = rp + RW;
-        const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
-        const uint32_t p1 = rp[j + 1], p2 = rp[j + 2];
-        const uint32_t q0 = rq[j], q1 = rq[j + 1];
-        tb = p1;
-        S = count_unlike(ta, Am, m1, fsr(m1, m2, 1), fsr(p1, p2, 1), q1, fsr(q0, q1, 31));
+        const uint32_t *pq = pp + RW;
+        tb = pp[0];
+        S = count_unlike(ta, Am, pm[0], window_p1(pm, E), window_p1(pp, E), pq[0], window_m1(pq, E));
     } else if (G == kTRI6 && OI == 2) {
         // a: (-1,0) (0,1) (-1,1); b = (1,-1): (2,-1) (1,-2) (2,-2); common (1,0) (0,-1)
-        const uint32_t *rn = rm - RW;
-        const uint32_t n1 = rn[j + 1], n2 = rn[j + 2];
-        const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
-        const uint32_t p0 = rp[j], p1 = rp[j + 1];
-        tb = fsr(m1, m2, 1);
-        S = count_unlike(ta, Am, p1, fsr(p0, p1, 31), fsr(m1, m2, 2), fsr(n1, n2, 1), fsr(n1, n2, 2));
+        const uint32_t *pn = pm - RW;
+        tb = window_p1(pm, E);
+        S = count_unlike(ta, Am, pp[0], window_m1(pp, E), window_p2<FIX>(pm, E), window_p1(pn, E), window_p2<FIX>(pn, E));
     } else if (G == kSQ4 && OI == 0) {
         // a: (-1,0) (0,1) (0,-1); b = (1,0): (2,0) (1,1) (1,-1)
-        const uint32_t a2 = r0[j + 2];
-        const uint32_t m1 = rm[j + 1], m2 = rm[j + 2];
-        const uint32_t p1 = rp[j + 1], p2 = rp[j + 2];
-        tb = fsr(a1, a2, 1);
-        S = count_unlike(ta, Am, p1, m1, fsr(a1, a2, 2), fsr(p1, p2, 1), fsr(m1, m2, 1));
+        tb = window_p1(p, E);
+        S = count_unlike(ta, Am, pp[0], pm[0], window_p2<FIX>(p, E), window_p1(pp, E), window_p1(pm, E));
     } else {
         // SQ4; a: (1,0) (-1,0) (0,-1); b = (0,1): (1,1) (-1,1) (0,2)
-        const uint32_t *rq = rp + RW;
-        const uint32_t a2 = r0[j + 2];
-        const uint32_t p0 = rp[j], p1 = rp[j + 1], p2 = rp[j + 2];
-        tb = p1;
-        S = count_unlike(ta, fsr(a1, a2, 1), Am, rm[j + 1], fsr(p1, p2, 1), fsr(p0, p1, 31), rq[j + 1]);
+        tb = pp[0];
+        S = count_unlike(ta, window_p1(p, E), Am, pm[0], window_p1(pp, E), window_m1(pp, E), pp[RW]);
     }
 }
 
+// Partners b = a + o of the accepted anchors acc of a word with ends E: their mask in
+// the word at the same place of b's row, and (returned) the one that falls into the
+// word on its right, as its bit 0.
+template <int OI>
+__device__ __forceinline__ uint32_t partners(uint32_t acc, const WordEnds &E, uint32_t &b)
+{
+    if (OI == 1) {
+        b = acc;
+        return 0u;
+    }
+    b = (acc << 1) & (2u * (1u << E.end) - 1u);
+    return (acc >> E.end) & 1u;
+}
+
 // Accept bits of the positions in dmask, each drawing Philox word 0 of counter
-// {site_base + p, f, s_lo, s_hi}; two evaluations interleaved at a time.
-__device__ __forceinline__ uint32_t draw_accepts(uint32_t dmask, const Planes &S,
-                                                 uint32_t site_base, const DrawKey &dk,
-                                                 const uint64_t *thr)
+// {site_base + p, f, s_lo, s_hi}; two evaluations interleaved at a time (after an odd
+// last draw the second one's bit is 0).  The first two are drawn without a test for
+// any: nearly every warp has a lane that needs them, and without the branch they are
+// scheduled into the evaluation.  The round keys are added up in every draw: sixteen
+// registers of them cost more than the additions.  (400^2 on 16 CTAs: 1.32 -> 1.18 us
+// per phase; 256 uneven replicas on 128 threads per CTA: 177 -> 162 us per sweep.)
+__device__ __forceinline__ uint32_t draw_accepts(uint32_t dmask, const Planes &S, uint32_t site_base,
+                                                 const DrawKey &dk, const DrawThr &T)
 {
     uint32_t acc = 0u;
     uint32_t dm = dmask;
-    while (dm != 0u) {
-        const int p1 = __ffs(dm) - 1;
-        dm &= dm - 1u;
-        const int p2 = dm != 0u ? __ffs(dm) - 1 : p1;  // an odd last draw is repeated
-        dm &= dm - 1u;
+    do {
+        const uint32_t b1 = dm & (0u - dm);
+        dm ^= b1;
+        const uint32_t b2 = dm & (0u - dm);
+        dm ^= b2;
         uint32_t r1, r2;
-        philox2_w0_key(site_base + (uint32_t)p1, site_base + (uint32_t)p2, dk, r1, r2);
-        if ((uint64_t)r1 < thr[plane_bits(S, p1)]) acc |= 1u << p1;
-        if ((uint64_t)r2 < thr[plane_bits(S, p2)]) acc |= 1u << p2;
-    }
-    return acc;
+        philox2_w0_key(site_base + (uint32_t)bit_index(b1), site_base + (uint32_t)bit_index(b2), dk, r1, r2);
+        if (accepts(r1, S.s0, S.s1, b1, T.t)) acc |= b1;
+        if (accepts(r2, S.s0, S.s1, b2, T.t)) acc |= b2;
+    } while (dm != 0u);
+    return acc & ~never_accepted(S.s0, S.s1, T.never);
 }
 
 // Accept bits of two tasks per lane (t and t + THREADS) when the warp's draws are
@@ -291,22 +360,23 @@ __device__ __forceinline__ uint32_t draw_accepts(uint32_t dmask, const Planes &S
 // shared atomics.  One scan and one pass serve both tasks, so a pass drains about
 // twice the draws of one task per lane.  When the warp has more than kDrawQueue2
 // draws, each lane draws its own.  Every lane of the warp must call it.  Region q
-// (16-byte aligned, kDrawQueue2Words words): records uint4[2][32] (the three planes
-// and the first site), accept words uint32[2][32] (zero on entry and on return),
+// (16-byte aligned, kDrawQueue2Words words): records uint4[2][32] (the two low planes
+// of S and the first site), accept words uint32[2][32] (zero on entry and on return),
 // entries uint16[kDrawQueue2].
 constexpr int kDrawQueue2 = 512;
 constexpr int kDrawQueue2Acc = 2 * 32 * 4;  // word offset of the accept words
 constexpr int kDrawQueue2Words = kDrawQueue2Acc + 2 * 32 + kDrawQueue2 / 2;
 
-template <bool RK>  // RK: the round keys from rk (kernel parameter space); else from dk
 __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Planes &S0, uint32_t base0,
                                                     uint32_t dmask1, const Planes &S1, uint32_t base1,
                                                     const DrawKey &dk, const uint32_t (&rk)[2][8],
-                                                    const uint64_t *thr, uint32_t *q, uint32_t &acc0,
+                                                    const DrawThr &T, uint32_t *q, uint32_t &acc0,
                                                     uint32_t &acc1)
 {
     acc0 = 0u;
     acc1 = 0u;
+    dmask0 &= ~never_accepted(S0.s0, S0.s1, T.never);
+    dmask1 &= ~never_accepted(S1.s0, S1.s1, T.never);
     if (!__any_sync(0xFFFFFFFFu, (dmask0 | dmask1) != 0u)) return;
     const int lane = (int)(threadIdx.x & 31);
     const int nd0 = __popc(dmask0), nd = nd0 + __popc(dmask1);
@@ -318,15 +388,15 @@ __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Plane
     }
     const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
     if (total > kDrawQueue2) {
-        acc0 = draw_accepts(dmask0, S0, base0, dk, thr);
-        acc1 = draw_accepts(dmask1, S1, base1, dk, thr);
+        acc0 = draw_accepts(dmask0, S0, base0, dk, T);
+        acc1 = draw_accepts(dmask1, S1, base1, dk, T);
         return;
     }
     uint4 *const rec = (uint4 *)q;  // [2][32]
     uint32_t *const wacc = q + kDrawQueue2Acc;  // [2][32]
     uint16_t *const ent = (uint16_t *)(wacc + 64);
-    if (dmask0 != 0u) rec[lane] = make_uint4(S0.s0, S0.s1, S0.s2, base0);
-    if (dmask1 != 0u) rec[32 + lane] = make_uint4(S1.s0, S1.s1, S1.s2, base1);
+    if (dmask0 != 0u) rec[lane] = make_uint4(S0.s0, S0.s1, base0, 0u);
+    if (dmask1 != 0u) rec[32 + lane] = make_uint4(S1.s0, S1.s1, base1, 0u);
     int slot = incl - nd;
     uint32_t dm = dmask0;
     while (dm != 0u) {
@@ -352,16 +422,15 @@ __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Plane
             const uint32_t r1i = e1 >> 5, p1 = e1 & 31u, r2i = e2 >> 5, p2 = e2 & 31u;  // record = task*32 + lane
             const uint4 a = rec[r1i], b = rec[r2i];
             uint32_t r1, r2;
-            if (RK) philox2_w0_rk(a.w + p1, b.w + p2, dk, rk, r1, r2);
-            else philox2_w0_key(a.w + p1, b.w + p2, dk, r1, r2);
-            if ((uint64_t)r1 < thr[plane_bits({a.x, a.y, a.z}, (int)p1)]) atomicOr(wacc + r1i, 1u << p1);
-            if (two && (uint64_t)r2 < thr[plane_bits({b.x, b.y, b.z}, (int)p2)]) atomicOr(wacc + r2i, 1u << p2);
+            philox2_w0_rk(a.z + p1, b.z + p2, dk, rk, r1, r2);
+            if (accepts(r1, a.x, a.y, 1u << p1, T.t)) atomicOr(wacc + r1i, 1u << p1);
+            if (two && accepts(r2, b.x, b.y, 1u << p2, T.t)) atomicOr(wacc + r2i, 1u << p2);
         } else if (k < total) {
             const uint32_t e1 = ent[k];
             const uint32_t r1i = e1 >> 5, p1 = e1 & 31u;
             const uint4 a = rec[r1i];
-            const uint32_t r1 = RK ? philox_w0_rk(a.w + p1, dk, rk) : philox_w0_key(a.w + p1, dk);
-            if ((uint64_t)r1 < thr[plane_bits({a.x, a.y, a.z}, (int)p1)]) atomicOr(wacc + r1i, 1u << p1);
+            const uint32_t r1 = philox_w0_rk(a.z + p1, dk, rk);
+            if (accepts(r1, a.x, a.y, 1u << p1, T.t)) atomicOr(wacc + r1i, 1u << p1);
         }
     }
     __syncwarp();
@@ -372,42 +441,46 @@ __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Plane
     __syncwarp();
 }
 
-// One padded shared-memory row from the device store (see the row layout above):
-// word 0 holds position -1 (site Lx-1) in bit 31; words 1..W hold sites 0..Lx-1;
-// positions Lx, Lx+1 hold sites 0, 1; every other pad bit is zero.
+// Word w (32 sites) of row y of the device store, the bits past the row's end zero.
 __device__ __forceinline__ uint32_t store_word(const void *lat, int packing, int pitch, int y, int w,
                                                int Lx)
 {
-    if (packing == kPackBit) return ((const uint32_t *)lat)[(size_t)y * pitch + w];
-    const uint8_t *row = (const uint8_t *)lat + (size_t)y * pitch + 32 * w;
     const int n = min(32, Lx - 32 * w);
+    if (packing == kPackBit) {
+        const uint32_t v = ((const uint32_t *)lat)[(size_t)y * pitch + w];
+        return n < 32 ? v & ((1u << n) - 1u) : v;
+    }
+    // rows of a multiple of 16 bytes, zeros past the last site: four sites at a time
+    const uint8_t *const bytes = (const uint8_t *)lat + (size_t)y * pitch + 32 * w;
+    const uint32_t *const row = (const uint32_t *)bytes;
     uint32_t v = 0u;
-    for (int b = 0; b < n; ++b) v |= (row[b] ? 1u : 0u) << b;
-    return v;
+    if ((uintptr_t)bytes & 3u) {  // a caller's allocator
+        for (int b = 0; b < n; ++b) v |= (uint32_t)(bytes[b] & 1u) << b;
+        return v;
+    }
+    for (int q = 0; 4 * q < n; ++q) {
+        const uint32_t b = row[q];  // bytes of 0 or 1
+        v |= ((b & 1u) | ((b >> 7) & 2u) | ((b >> 14) & 4u) | ((b >> 21) & 8u)) << (4 * q);
+    }
+    return n < 32 ? v & ((1u << n) - 1u) : v;
 }
 
-__device__ __forceinline__ uint32_t padded_word(const void *lat, int packing, int pitch, int y,
-                                                int w, int Lx, int W)
+// Writes word w of row y to the device store (sites only).
+__device__ __forceinline__ void write_word(void *lat, int packing, int pitch, int y, int w, int Lx, uint32_t v)
 {
-    const int P0 = 32 * w - 32;  // first position held by word w
-    uint32_t v = 0u;
-    if (w >= 1 && w <= W) {
-        v = store_word(lat, packing, pitch, y, w - 1, Lx);
-        const int nvalid = Lx - P0;
-        if (nvalid < 32) v &= (1u << nvalid) - 1u;
+    if (packing == kPackBit) {
+        ((uint32_t *)lat)[(size_t)y * pitch + w] = v;
+        return;
     }
-    if (w == 0) {
-        const int xl = Lx - 1;
-        v |= ((store_word(lat, packing, pitch, y, xl >> 5, Lx) >> (xl & 31)) & 1u) << 31;
+    const int n = min(32, Lx - 32 * w);
+    uint8_t *const bytes = (uint8_t *)lat + (size_t)y * pitch + 32 * w;
+    uint32_t *const row = (uint32_t *)bytes;
+    if ((uintptr_t)bytes & 3u) {  // a caller's allocator
+        for (int b = 0; b < n; ++b) bytes[b] = (uint8_t)((v >> b) & 1u);
+        return;
     }
-    const int q0 = Lx - P0;  // bit of position Lx in this word
-    if (q0 >= -1 && q0 < 32) {
-        const uint32_t s01 = store_word(lat, packing, pitch, y, 0, Lx) & 3u;  // sites 0, 1
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int q = q0 + e;
-            if (q >= 0 && q < 32) v |= ((s01 >> e) & 1u) << q;
-        }
+    for (int q = 0; 4 * q < n; ++q) {
+        const uint32_t b = v >> (4 * q);
+        row[q] = (b & 1u) | ((b & 2u) << 7) | ((b & 4u) << 14) | ((b & 8u) << 21);
     }
-    return v;
 }

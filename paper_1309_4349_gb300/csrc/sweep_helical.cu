@@ -95,96 +95,11 @@ __host__ __device__ __forceinline__ int helical_block(int Lx, int Ly, int C)
 }
 
 struct HGeo {
-    int Lx, Ly, W, RW, D, H, Y0, C, rank, sign, NL;
+    int Lx, Ly, W, RW, D, H, Y0, C, rank, sign, NL, nlast;
     long long N;
     unsigned long long magicW;
     uint32_t k0, k1, lat_addr;
 };
-
-// Word w of the padded row of global row y: positions [32 w - 32, 32 w); position
-// p holds site (y Lx + p) mod N.  Only positions -1 .. Lx + 1 are ever read.
-__device__ __forceinline__ uint32_t helical_word(const SweepJob &J, int y, int w)
-{
-    const int Lx = J.Lx, Ly = J.Ly, W = J.W;
-    const int P0 = 32 * w - 32;
-    uint32_t v = 0u;
-    if (w >= 1 && w <= W) {
-        v = store_word(J.lat, J.packing, J.pitch, y, w - 1, Lx);
-        const int nvalid = Lx - P0;
-        if (nvalid < 32) v &= (1u << nvalid) - 1u;
-    }
-    if (w == 0) {  // position -1: the last site of row y - 1
-        const int yp = y == 0 ? Ly - 1 : y - 1;
-        const int xl = Lx - 1;
-        v |= ((store_word(J.lat, J.packing, J.pitch, yp, xl >> 5, Lx) >> (xl & 31)) & 1u) << 31;
-    }
-    const int q0 = Lx - P0;  // bit of position Lx in this word
-    if (q0 >= -1 && q0 < 32) {
-        const int yn = y + 1 == Ly ? 0 : y + 1;
-        const uint32_t s01 = store_word(J.lat, J.packing, J.pitch, yn, 0, Lx) & 3u;  // sites 0, 1 of row y + 1
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int q = q0 + e;
-            if (q >= 0 && q < 32) v |= ((s01 >> e) & 1u) << q;
-        }
-    }
-    return v;
-}
-
-// Sets padded position pos of local row lr to bit b (plain store: one thread per row).
-__device__ __forceinline__ void set_position(uint32_t *lat, int RW, int lr, int pos, uint32_t b)
-{
-    uint32_t *row = lat + (size_t)lr * RW;
-    const int w = (pos + 32) >> 5, s = (pos + 32) & 31;
-    row[w] = (row[w] & ~(1u << s)) | (b << s);
-}
-
-// Recomputes the pads of local rows [lo, hi) from the rows beside them.
-__device__ __forceinline__ void helical_pads(uint32_t *lat, const HGeo &g, int lo, int hi)
-{
-    for (int lr = lo + (int)threadIdx.x; lr < hi; lr += kHelicalThreads) {
-        if (lr >= 1) {
-            const uint32_t *up = lat + (size_t)(lr - 1) * g.RW;
-            const int xl = g.Lx - 1;
-            set_position(lat, g.RW, lr, -1, (up[(xl >> 5) + 1] >> (xl & 31)) & 1u);
-        }
-        if (lr + 1 < g.NL) {
-            const uint32_t s01 = lat[(size_t)(lr + 1) * g.RW + 1] & 3u;
-            set_position(lat, g.RW, lr, g.Lx, s01 & 1u);
-            set_position(lat, g.RW, lr, g.Lx + 1, s01 >> 1);
-        }
-    }
-}
-
-// XOR mask into padded positions q .. q+31 of the local row at shared address row.
-__device__ __forceinline__ void hxor_at(uint32_t row, int RW, int q, uint32_t mask)
-{
-    if (mask == 0u) return;
-    if (q < 0) {
-        if (q <= -32) return;
-        mask >>= -q;
-        q = 0;
-    }
-    const int w = q >> 5, s = q & 31;
-    if (w < RW) hred_xor(row + 4u * w, mask << s);
-    if (s != 0 && w + 1 < RW) hred_xor(row + 4u * (w + 1), mask >> (32 - s));
-}
-
-// Flips, in local row lr, the sites x0 + i (bit i of m, x0 = 32 j, every site < Lx),
-// and their copies in the pads of the rows above and below (when held).
-__device__ __forceinline__ void helical_flip(const HGeo &g, int lr, int j, unsigned long long m)
-{
-    if (m == 0ull) return;
-    const uint32_t rowbytes = 4u * (uint32_t)g.RW;
-    const uint32_t row = g.lat_addr + rowbytes * (uint32_t)lr;
-    const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32);
-    if (lo) hred_xor(row + 4u * (uint32_t)(j + 1), lo);
-    if (hi) hred_xor(row + 4u * (uint32_t)(j + 2), hi);
-    if (j == 0 && (lo & 3u) && lr >= 1)  // sites 0, 1: positions Lx, Lx + 1 of the row above
-        hxor_at(row - rowbytes, g.RW, g.Lx + 32, lo & 3u);
-    const int b = g.Lx - 1 - 32 * j;  // site Lx - 1: position -1 of the row below
-    if (b >= 0 && b < 64 && ((m >> b) & 1ull) && lr + 1 < g.NL) hred_xor(row + rowbytes, 0x80000000u);
-}
 
 struct HAcc {
     uint32_t unl, drw, acc;
@@ -196,36 +111,35 @@ struct HAcc {
 // cluster's shared memory has far fewer than 2^30 sites, and base lies within
 // [-Lx, N + Lx).
 __device__ __forceinline__ uint32_t helical_draws(uint32_t dmask, const Planes &S, int base, int N,
-                                                  const DrawKey &dk, const uint64_t *thr)
+                                                  const DrawKey &dk, const DrawThr &T)
 {
     uint32_t acc = 0u;
     uint32_t dm = dmask;
-    while (dm != 0u) {
-        const int p1 = __ffs(dm) - 1;
-        dm &= dm - 1u;
-        const int p2 = dm != 0u ? __ffs(dm) - 1 : p1;  // an odd last draw is repeated
-        dm &= dm - 1u;
-        int c1 = base + p1, c2 = base + p2;
+    do {
+        const uint32_t b1 = dm & (0u - dm);
+        dm ^= b1;
+        const uint32_t b2 = dm & (0u - dm);  // 0 after an odd last draw
+        dm ^= b2;
+        int c1 = base + bit_index(b1), c2 = base + bit_index(b2);
         c1 += c1 >= N ? -N : (c1 < 0 ? N : 0);
         c2 += c2 >= N ? -N : (c2 < 0 ? N : 0);
         uint32_t r1, r2;
         philox2_w0_key((uint32_t)c1, (uint32_t)c2, dk, r1, r2);
-        if ((uint64_t)r1 < thr[plane_bits(S, p1)]) acc |= 1u << p1;
-        if ((uint64_t)r2 < thr[plane_bits(S, p2)]) acc |= 1u << p2;
-    }
-    return acc;
+        if (accepts(r1, S.s0, S.s1, b1, T.t)) acc |= b1;
+        if (accepts(r2, S.s0, S.s1, b2, T.t)) acc |= b2;
+    } while (dm != 0u);
+    return acc & ~never_accepted(S.s0, S.s1, T.never);
 }
 
 // One iteration: anchors of residue kr mod 7 in local rows [lr0, lr0 + nrows),
 // orientation OI, draw counters shifted by delta (the centre of a backward pair).
 template <int OI>
 __device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGeo &g, int kr, int delta,
-                                                  int lr0, int nrows, const DrawKey &dk, const uint64_t *thr,
-                                                  HAcc &A)
+                                                  int lr0, int nrows, const DrawKey &dk,
+                                                  const DrawThr &T, HAcc &A)
 {
     // b = a + o: (1,0) -> same row, +1; (0,1) -> next row; (1,-1) -> previous row, +1
-    constexpr int bdy = OI == 0 ? 0 : (OI == 1 ? 1 : -1);
-    constexpr int bdx = OI == 1 ? 0 : 1;
+    const uint32_t rowbytes = 4u * (uint32_t)g.RW;
     const int ntask = nrows * g.W;
     for (int t = (int)threadIdx.x; t < ntask; t += kHelicalThreads) {
         const int mi = (int)(((unsigned long long)t * g.magicW) >> 32);
@@ -242,11 +156,12 @@ __device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGe
         if (g.Lx - x0 < 32) am &= (1u << (g.Lx - x0)) - 1u;
         uint32_t ta, tb;
         Planes S;
-        evaluate<kTRI6, OI>(lat + (size_t)lr * g.RW, g.RW, j, ta, tb, S);
+        const WordEnds E = word_ends(j, g.W, g.nlast, g.RW);
+        evaluate<kTRI6, OI, true>(lat + lr * g.RW + j, g.RW, E, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
         const uint32_t dmask = unl & draw_positions(S, g.sign);
         uint32_t acc = unl & ~dmask;
-        acc |= helical_draws(dmask, S, (int)a0 + delta, (int)g.N, dk, thr);
+        acc |= helical_draws(dmask, S, (int)a0 + delta, (int)g.N, dk, T);
         const bool own = (unsigned)(lr - g.D) < (unsigned)g.H;
         if (own) {
             A.unl += __popc(unl);
@@ -258,24 +173,17 @@ __device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGe
             A.acc += na;
             A.dn += 2 * half_dn(S, acc, na);
         }
-        // b sites; with bdx = 1 the partner of anchor Lx-1 is position Lx, site 0 of
-        // the next row of the b row.
-        unsigned long long mb = (unsigned long long)acc << bdx;
-        bool wrap0 = false;
-        if (bdx == 1) {
-            const int wb = g.Lx - x0;
-            if (wb <= 32 && ((mb >> wb) & 1ull)) {
-                mb &= ~(1ull << wb);
-                wrap0 = true;
-            }
-        }
-        if (bdy == 0) {
-            helical_flip(g, lr, j, (unsigned long long)acc | mb);
+        const uint32_t wa = g.lat_addr + 4u * (uint32_t)(lr * g.RW + j);
+        const uint32_t wb = OI == 0 ? wa : (OI == 1 ? wa + rowbytes : wa - rowbytes);
+        uint32_t b;
+        const uint32_t next = partners<OI>(acc, E, b);
+        if (OI == 0) {
+            hred_xor(wa, acc | b);
         } else {
-            helical_flip(g, lr, j, (unsigned long long)acc);
-            helical_flip(g, lr + bdy, j, mb);
+            hred_xor(wa, acc);
+            hred_xor(wb, b);
         }
-        if (wrap0) helical_flip(g, lr + bdy + 1, 0, 1ull);
+        if (OI != 1) hred_xor(wb + 4u * (uint32_t)E.r, next);
     }
 }
 
@@ -292,7 +200,6 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
 {
     constexpr int kWarps = kHelicalThreads / 32;
     extern __shared__ __align__(16) uint32_t lat[];
-    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
     __shared__ uint2 sched[2];  // (colour, direction draw) of the current and the next iteration
     if (Cl.n_mcs <= 0) return;
@@ -301,6 +208,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = J.RW; g.magicW = J.magicW;
     g.k0 = J.key0; g.k1 = J.key1;
     g.N = (long long)J.Lx * J.Ly;
+    g.nlast = g.Lx - 32 * (g.W - 1);
     // The host's draw range is [z, 2(z-1)] (omega > 0), [0, z-2] (omega < 0) or empty.
     g.sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
     g.C = (int)hcluster_nctarank();
@@ -319,9 +227,9 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
         const int lr = idx / g.RW, w = idx - lr * g.RW;
         int y = (g.Y0 - g.D + lr) % g.Ly;
         if (y < 0) y += g.Ly;
-        lat[idx] = helical_word(J, y, w);
+        lat[idx] = w < g.W ? store_word(J.lat, J.packing, J.pitch, y, w, g.Lx) : 0u;
     }
-    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
+    const DrawThr T = draw_thresholds(J);
     // Iteration f of sweep s draws its colour and direction from one Philox block;
     // the last warp's lane 0 draws them one iteration ahead, off the tasks' path.
     const bool sched_lane = tid == kHelicalThreads - 32;
@@ -357,9 +265,9 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
                 sched[pb ^ 1] = f == 6 ? helical_sched(g, (unsigned long long)(s + 1), 0)
                                        : helical_sched(g, (unsigned long long)s, f + 1);
             const DrawKey dk = draw_key((uint32_t)f, s_lo, s_hi, g.k0, g.k1);
-            if (oi == 0) helical_iteration<0>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, thr, A);
-            else if (oi == 1) helical_iteration<1>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, thr, A);
-            else helical_iteration<2>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, thr, A);
+            if (oi == 0) helical_iteration<0>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, T, A);
+            else if (oi == 1) helical_iteration<1>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, T, A);
+            else helical_iteration<2>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, T, A);
             __syncthreads();
             pb ^= 1;
             const bool last = f == 6 && it + 1 == Cl.n_mcs;
@@ -390,8 +298,6 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
                     lat[(size_t)(side ? g.D + g.H : 0) * g.RW + k] = mbox[(size_t)(2 * p + side) * rw + k];
                 }
                 __syncthreads();
-                helical_pads(lat, g, 0, g.NL);
-                __syncthreads();
                 ++block;
             }
         }
@@ -411,16 +317,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     for (int idx = tid; idx < g.H * g.W; idx += kHelicalThreads) {
         const int r = idx / g.W, w = idx - r * g.W;
         const int y = g.Y0 + r;
-        const uint32_t v = lat[(size_t)(r + g.D) * g.RW + w + 1];
-        const int pos0 = 32 * w;
-        const int nvalid = min(32, g.Lx - pos0);
-        if (J.packing == kPackBit) {
-            const uint32_t valid = nvalid == 32 ? 0xFFFFFFFFu : ((1u << nvalid) - 1u);
-            ((uint32_t *)J.lat)[(size_t)y * J.pitch + w] = v & valid;
-        } else {
-            uint8_t *row = (uint8_t *)J.lat + (size_t)y * J.pitch;
-            for (int b = 0; b < nvalid; ++b) row[pos0 + b] = (uint8_t)((v >> b) & 1u);
-        }
+        write_word(J.lat, J.packing, J.pitch, y, w, g.Lx, lat[(r + g.D) * g.RW + w]);
     }
 
     long long vals[5] = {(long long)t_att, (long long)t_unl, (long long)t_drw, (long long)t_acc, t_dn};

@@ -14,7 +14,7 @@
 // a cluster barrier (release/acquire), so the next phase sees every flip.
 //
 // Phase blocks.  When the bands are tall enough, a cluster of C > 1 CTAs instead
-// advances K consecutive phases (K = 2, 4 or 8) between exchanges.  Each CTA
+// advances K consecutive phases (K = 2 or 4) between exchanges.  Each CTA
 // keeps D = 2K + 1 halo rows on each side, and in the j-th phase of a block
 // evaluates every anchor within 2 (K - 1 - j) + 1 rows of its band: a site's new
 // value depends only on sites at most two rows away, so after K phases the band
@@ -23,15 +23,12 @@
 // random numbers, hence identical results; only anchors of the own band are
 // counted.  All flips are local.  At the end of a block each CTA stores its D
 // lowest and D highest band rows into mailboxes in the neighbouring CTAs'
-// shared memory (double-buffered by block parity), one cluster barrier follows,
-// and each CTA copies its mailboxes into its halo rows.
+// shared memory (double-buffered by block parity) and waits for its own two
+// neighbours' rows, which it copies into its halo rows.
 //
-// Row layout.  A shared-memory row is RW 32-bit words holding the padded bit
-// positions pos in [-32, 32*RW - 32); when loaded, position pos holds site
-// (pos mod Lx), so the 32-site window starting at any x in [-32, Lx + 32] is one
-// funnel shift of two words.  The windows of anchors x < Lx read only positions
-// -1 .. Lx+1, so flips keep exactly the copies at -1 (site Lx-1) and Lx, Lx+1
-// (sites 0, 1) equal to their sites; other pad positions are never read.
+// Row layout.  A shared-memory row is W words of 32 sites at a stride of RW = W + 2
+// words, the bits of the last word past the row's end zero.  The windows of the
+// words at a row's ends reach around them (WordEnds in sweep_common.cuh).
 //
 // Evaluation.  One thread handles the anchors of one 32-site word of one anchor
 // row.  Neighbour comparisons of all 32 positions are bitwise operations summed by
@@ -43,6 +40,8 @@
 // lane draws for its own anchors, two Philox evaluations interleaved at a time:
 // a phase is short, so its cost is the latency of its slowest task.
 #include <string.h>
+
+#include <type_traits>
 
 #include "klmc_internal.h"
 #include "philox.cuh"
@@ -76,29 +75,16 @@ __device__ __forceinline__ void red_xor_local(uint32_t addr, uint32_t v)
     asm volatile("red.shared.xor.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// XOR mask into padded bit positions q .. q+31 of the row at shared address row (clipped).
-__device__ __forceinline__ void xor_at(uint32_t row, int RW, int q, uint32_t mask, uint32_t rank,
-                                       bool local)
-{
-    if (q < 0) {
-        if (q <= -32) return;
-        mask >>= -q;
-        q = 0;
-    }
-    const int w = q >> 5, s = q & 31;
-    if (w < RW) xor_word(row + 4u * w, rank, local, mask << s);
-    if (s != 0 && w + 1 < RW) xor_word(row + 4u * (w + 1), rank, local, mask >> (32 - s));
-}
-
 struct Acc {
     uint32_t unl, drw, acc;
-    int32_t dn;
+    int32_t dn;  // n_unlike change / 2
 };
 
 struct Geo {
     int Lx, Ly, W, RW;
-    unsigned long long magicW;
+    uint32_t magicW, one;  // task t is word t - m W of row m = (t magicW) >> 32 (W = 1: magicW 0, one ~0, m = t)
     uint32_t k0, k1;
+    bool tri;            // triangular (else square) geometry
     int sign;            // draw when the exchange raises (+1) / lowers (-1) E; 0: never
     int C, rank, Y0, Y1;
     int prevY, prevH;    // band of CTA rank-1 (mod C)
@@ -106,35 +92,47 @@ struct Geo {
     uint32_t lat_addr;   // shared address of local row 0
     int D;               // halo rows on each side: local row lr holds row (Y0 - D + lr) mod Ly
     int base;            // (Y0 - D) mod Ly
+    int tabW;            // words of a table's anchor masks (even)
+    int nlast;           // sites of a row's last word
 };
 
-// Flip, in one copy of a row, the sites x0 + i (bit i of m, x0 = 32 j, every site
-// < Lx), and the pad copies that windows read: position -1 (site Lx-1) and
-// positions Lx, Lx+1 (sites 0, 1).
-__device__ __forceinline__ void flip_row(const Geo &g, uint32_t row, int j, unsigned long long m,
-                                         uint32_t rank, bool local)
+__device__ __forceinline__ int task_row(const Geo &g, int t)
 {
-    const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32);
-    xor_word(row + 4u * (uint32_t)(j + 1), rank, local, lo);
-    xor_word(row + 4u * (uint32_t)(j + 2), rank, local, hi);
-    if (j == 0 && (lo & 3u)) xor_at(row, g.RW, g.Lx + 32, lo & 3u, rank, local);
-    const int b = g.Lx - 1 - 32 * j;
-    if (b >= 0 && b < 64 && ((m >> b) & 1ull)) xor_word(row, rank, local, 0x80000000u);
+    return (int)(__umulhi((uint32_t)t, g.magicW) + ((uint32_t)t & g.one));
 }
 
-// Flip sites of global row r (unwrapped, in [Y0 - 1, Y1]) in every CTA holding a copy.
-__device__ __forceinline__ void flip_global_row(const Geo &g, int r, int j, unsigned long long m)
+// Flips, in this CTA's rows, the accepted anchors acc of the word at shared address wa
+// and their partners.  Atomics of 0 cost less than branches around them.
+template <int OI>
+__device__ __forceinline__ void flip_pairs(uint32_t wa, int RW, const WordEnds &E, uint32_t acc)
 {
+    const uint32_t rowbytes = 4u * (uint32_t)RW;
+    const uint32_t wb = OI == 0 ? wa : (OI == 1 ? wa + rowbytes : wa - rowbytes);
+    uint32_t b;
+    const uint32_t next = partners<OI>(acc, E, b);
+    if (OI == 0) {
+        red_xor_local(wa, acc | b);
+    } else {
+        red_xor_local(wa, acc);
+        red_xor_local(wb, b);
+    }
+    if (OI != 1) red_xor_local(wb + 4u * (uint32_t)E.r, next);
+}
+
+// Flips m in word j of global row r (unwrapped, in [Y0 - 1, Y1]) in every CTA holding a copy.
+__device__ __forceinline__ void flip_global_row(const Geo &g, int r, int j, uint32_t m)
+{
+    if (m == 0u) return;
+    const uint32_t word = g.lat_addr + 4u * (uint32_t)j, rowbytes = 4u * (uint32_t)g.RW;
     const int lr_self = r - g.Y0 + 2;
-    const uint32_t rowbytes = 4u * (uint32_t)g.RW;
-    if (g.C > 1 && lr_self >= 4 && lr_self < g.Y1 - g.Y0) {  // interior row: local copy only
-        flip_row(g, g.lat_addr + rowbytes * (uint32_t)lr_self, j, m, 0u, true);
+    if (lr_self >= 4 && lr_self < g.Y1 - g.Y0) {  // interior row: local copy only
+        red_xor_local(word + rowbytes * (uint32_t)lr_self, m);
         return;
     }
     const int gr = r < 0 ? r + g.Ly : (r >= g.Ly ? r - g.Ly : r);
     if (g.C == 1) {  // rows 0, 1 and Ly-2, Ly-1 also live in the opposite halo
         for (int lr = gr + 2 >= g.Ly ? gr + 2 - g.Ly : gr + 2; lr < g.Ly + 4; lr += g.Ly)
-            flip_row(g, g.lat_addr + rowbytes * (uint32_t)lr, j, m, 0u, true);
+            red_xor_local(word + rowbytes * (uint32_t)lr, m);
         return;
     }
     for (int k = 0; k < 3; ++k) {
@@ -146,29 +144,31 @@ __device__ __forceinline__ void flip_global_row(const Geo &g, int r, int j, unsi
         int lr = gr - Yd + 2;
         if (lr < 0) lr += g.Ly;
         if (lr >= g.Ly) lr -= g.Ly;
-        for (; lr < Hd + 4; lr += g.Ly)
-            flip_row(g, g.lat_addr + rowbytes * (uint32_t)lr, j, m, (uint32_t)d, d == g.rank);
+        for (; lr < Hd + 4; lr += g.Ly) xor_word(word + rowbytes * (uint32_t)lr, (uint32_t)d, d == g.rank, m);
     }
 }
 
-__device__ __forceinline__ void phase_barrier(int C)
+__device__ __forceinline__ void cluster_barrier()
 {
-    if (C == 1) {
-        __syncthreads();
-    } else {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
+
+// Barrier of the CTA's first NT threads, which run the tasks.
+template <int NT>
+__device__ __forceinline__ void task_barrier()
+{
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+}
+
+// Barrier of the whole CTA, reached by different warps in different places.
+__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
 
 // Per-phase task table: the anchor mask of every word and, per task row mi, the
 // local row and the row's first site index, so that a task loads two entries
-// instead of recomputing them.  The resident kernel keeps two (current and next
-// phase) for bands of at most kTabW words per row and kTabRows anchor rows, built by
-// the CTA's last warp while the other warps run the current phase; the band kernel
-// builds one per phase of its block at launch.
-constexpr int kTabW = 64;
-constexpr int kTabRows = 128;
+// instead of recomputing them.  The resident kernel keeps two chunks of kChunk phases
+// (the current one and the next), the band kernel the phases of its block.
+constexpr int kChunk = 4;
 
 struct TaskTab {  // a table's storage and capacity
     uint32_t *am;
@@ -181,17 +181,14 @@ __device__ __forceinline__ bool table_fits(const Geo &g, const PhaseR &P, const 
     return g.W <= T.maxw && P.c[3] <= T.maxrows;
 }
 
-// Fills the table entries with index = lane0 mod step (all of them for lane0 = 0,
-// step = 1 per thread ... ), so that a warp (step 32) or a CTA (step THREADS)
-// builds it together: the anchor masks (AM), the rows (ROWS) or both.
-template <bool BLOCKED, bool AM = true, bool ROWS = true>
+// Fills the table entries with index = lane0 mod step, so that a warp (step 32) or a
+// CTA (step THREADS) builds it together.
+template <bool BLOCKED>
 __device__ __forceinline__ void build_task_table(const PhaseR &P, const Geo &g, const TaskTab &T, int lane0,
                                                  int step)
 {
     if (!table_fits(g, P, T)) return;
-    if (AM)
-        for (int j = lane0; j < g.W; j += step) T.am[j] = anchor_mask(j << 5, P, g.Lx);
-    if (ROWS)
+    for (int j = lane0; j < g.W; j += step) T.am[j] = anchor_mask(j << 5, P, g.Lx);
     for (int mi = lane0; mi < P.c[3]; mi += step) {
         const int m = mi < P.c[0] ? P.a[0] + mi
                     : (mi < P.c[1] ? P.a[1] + mi : (mi < P.c[2] ? P.a[2] + mi : P.a[3] + mi));
@@ -208,112 +205,117 @@ __device__ __forceinline__ void build_task_table(const PhaseR &P, const Geo &g, 
     }
 }
 
-// One phase of one band.  Every task is (anchor row, word j).  BLOCKED: the
-// anchors span the band and part of its halo, all flips are local, and only
-// anchors of the band are counted; otherwise the anchors are those of the band
-// and flips reach every copy of their rows.
-template <int G, int OI, int THREADS, bool BLOCKED>
-__device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, const PhaseR &P,
-                                          const uint64_t *thr, int f,
-                                          uint32_t s_lo, uint32_t s_hi, Acc &A, const TaskTab *tt = nullptr)
+#ifndef KLMC_SPLIT_LANES
+#define KLMC_SPLIT_LANES(NT) ((NT) > 256 ? 256 : (NT))
+#endif
+// What a phase's tasks need of its schedule entry, prepared with the task table.
+struct __align__(16) PhaseHdr {
+    int nlane;        // lanes with tasks: the phase's words, each split over 2^ls lanes
+    int code;         // orientation + 4 ls
+    uint32_t hk, la;  // the phase's part of the draw key
+};
+
+// Lanes per word (log2) of a phase of ntask words on NT threads.  A split word's
+// lanes all evaluate it and each keeps the anchors of its part, which divides the
+// draws (the longest step of a lane) among them.
+template <int NT>
+__device__ __forceinline__ int word_split(int ntask)
+{
+    constexpr int kLanes = KLMC_SPLIT_LANES(NT);
+    return 4 * ntask <= kLanes ? 2 : (2 * ntask <= kLanes ? 1 : 0);
+}
+
+// One task of a phase: the word at p of an anchor row in local row lr (word j of it),
+// the site index of its first site, its ends and its anchors.
+struct Task {
+    const uint32_t *p;
+    int j, lr;
+    uint32_t site, am;
+    WordEnds E;
+};
+
+template <bool BLOCKED>
+__device__ __forceinline__ Task load_task(const uint32_t *lat, const Geo &g, int tl, int ls, const PhaseR &P,
+                                          bool use_tab, const uint32_t *tab)
+{
+    Task k;
+    const int t = tl >> ls;
+    const int mi = task_row(g, t);
+    k.j = t - mi * g.W;
+    int ybase;
+    if (use_tab) {
+        k.am = tab[k.j];
+        const int2 r = *(const int2 *)(tab + g.tabW + 2 * mi);
+        k.lr = r.x;
+        ybase = r.y;
+    } else {
+        const int m = mi < P.c[0] ? P.a[0] + mi
+                    : (mi < P.c[1] ? P.a[1] + mi : (mi < P.c[2] ? P.a[2] + mi : P.a[3] + mi));
+        int y = P.ry + P.py * m;
+        if (y >= g.Ly) y -= g.Ly;
+        if (BLOCKED) {
+            k.lr = y - g.base;
+            if (k.lr < 0) k.lr += g.Ly;
+        } else {
+            k.lr = y - g.Y0 + 2;  // y is a band row
+        }
+        ybase = y * g.Lx;
+        k.am = anchor_mask(k.j << 5, P, g.Lx);
+    }
+    // a split word's part (the thread count is a multiple of 4, so a thread's part is fixed)
+    const int bits = 32 >> ls;
+    k.am &= (0xFFFFFFFFu >> (32 - bits)) << ((tl & ((1 << ls) - 1)) * bits);
+    k.site = (uint32_t)(ybase + (k.j << 5));
+    k.p = lat + k.lr * g.RW + k.j;
+    k.E = word_ends(k.j, g.W, g.nlast, 0);
+    return k;
+}
+
+// One phase of one band, by the first NT threads of the CTA, the thread's first task
+// already loaded.  Every task is (anchor row, word j).  BLOCKED: the anchors span the
+// band and part of its halo, all flips are local, and only anchors of the band are
+// counted; otherwise the anchors are those of the band and flips reach every copy of
+// their rows.
+//
+// Bound: a warp issues an instruction about every five cycles (dependent operations
+// of one or two warps per scheduler), so a phase lasts as long as the instruction
+// stream of its busiest warp.  Branches in it cost most: the geometry, the orientation
+// and the rare row shapes are template parameters.
+template <int G, int OI, int NT, bool BLOCKED, bool FIX>
+__device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, const PhaseHdr &h, Task k,
+                                          const PhaseR &P, const DrawThr &T, const DrawKey &dk, Acc &A,
+                                          bool use_tab, const uint32_t *tab)
 {
     // b = a + o: (1,0) -> same row, +1; (0,1) -> next row; (1,-1) -> previous row, +1
     constexpr int bdy = OI == 0 ? 0 : (OI == 1 ? 1 : -1);
-    constexpr int bdx = OI == 1 ? 0 : 1;
-    const int lane = threadIdx.x & 31;
     const int H = g.Y1 - g.Y0;
-    // Split each word over 2^ls lanes when the phase has that few words: every lane
-    // evaluates the word and keeps the anchors of its part, which divides the draws
-    // (the longest step of a lane) among the lanes.
-    // (At 512 threads the extra evaluations cost more issue slots than they save.)
-    const int ls = THREADS > 256 ? 0 : (4 * P.ntask <= THREADS ? 2 : (2 * P.ntask <= THREADS ? 1 : 0));
-    const int nlane = P.ntask << ls;
-    const bool use_tab = tt != nullptr && table_fits(g, P, *tt);
-    const DrawKey dk = draw_key((uint32_t)f, s_lo, s_hi, g.k0, g.k1);
-    for (int t0 = threadIdx.x & ~31; t0 < nlane; t0 += THREADS) {
-        const int tl = t0 + lane;
-        uint32_t am = 0u, ta = 0u, tb = 0u;
-        Planes S = {0u, 0u, 0u};
-        int ybase = 0, x0 = 0, lr = 0;
-        if (tl < nlane) {
-            const int t = tl >> ls;
-            const int mi = (int)(((unsigned long long)t * g.magicW) >> 32);
-            const int j = t - mi * g.W;
-            x0 = j << 5;
-            if (use_tab) {
-                const int2 r = tt->row[mi];
-                lr = r.x;
-                ybase = r.y;
-                am = tt->am[j];
-            } else {
-                const int m = mi < P.c[0] ? P.a[0] + mi
-                            : (mi < P.c[1] ? P.a[1] + mi : (mi < P.c[2] ? P.a[2] + mi : P.a[3] + mi));
-                int y = P.ry + P.py * m;
-                if (y >= g.Ly) y -= g.Ly;
-                if (BLOCKED) {
-                    lr = y - g.base;
-                    if (lr < 0) lr += g.Ly;
-                } else {
-                    lr = y - g.Y0 + 2;  // y is a band row
-                }
-                ybase = y * g.Lx;
-                am = anchor_mask(x0, P, g.Lx);
-            }
-            if (ls != 0) {
-                const int part = tl & ((1 << ls) - 1), bits = 32 >> ls;
-                am &= (0xFFFFFFFFu >> (32 - bits)) << (part * bits);
-            }
-            evaluate<G, OI>(lat + (size_t)lr * g.RW, g.RW, j, ta, tb, S);
-        }
-        const uint32_t unl = (ta ^ tb) & am;
+    for (int tl = threadIdx.x; tl < h.nlane;) {
+        uint32_t ta, tb;
+        Planes S;
+        evaluate<G, OI, FIX>(k.p, g.RW, k.E, ta, tb, S);
+        const uint32_t unl = (ta ^ tb) & k.am;
         const uint32_t dmask = unl & draw_positions(S, g.sign);
-        uint32_t acc = unl & ~dmask;
-
-        acc |= draw_accepts(dmask, S, (uint32_t)(ybase + x0), dk, thr);
-        const bool own = !BLOCKED || (unsigned)(lr - g.D) < (unsigned)H;
-        if (own) {
-            A.unl += __popc(unl);
-            A.drw += __popc(dmask);
+        const uint32_t acc = (unl & ~dmask) | draw_accepts(dmask, S, k.site, dk, T);
+        const uint32_t own = !BLOCKED || (unsigned)(k.lr - g.D) < (unsigned)H ? ~0u : 0u;
+        const uint32_t oacc = acc & own;
+        const int na = __popc(oacc);
+        A.unl += __popc(unl & own);
+        A.drw += __popc(dmask & own);
+        A.acc += na;
+        A.dn += half_dn(S, oacc, na);
+        // One CTA: rows 2 .. Ly-3 have no copy in a halo.
+        if (BLOCKED || (g.C == 1 && k.lr >= 5 && k.lr < H - 1)) {
+            flip_pairs<OI>(smem_addr(k.p), g.RW, k.E, acc);
+        } else {
+            const int yu = k.lr - g.D + g.Y0;  // unwrapped band row
+            uint32_t b;
+            const uint32_t next = partners<OI>(acc, k.E, b);
+            flip_global_row(g, yu, k.j, acc);
+            flip_global_row(g, yu + bdy, k.j, b);
+            flip_global_row(g, yu + bdy, k.j + k.E.r, next);
         }
-        if (acc) {
-            if (own) {
-                const int na = __popc(acc);
-                A.acc += na;
-                A.dn += 2 * half_dn(S, acc, na);
-            }
-            const int j = x0 >> 5;
-            // b sites; with bdx = 1 the pair of anchor Lx-1 wraps to site 0.
-            unsigned long long mb = (unsigned long long)acc << bdx;
-            bool wrap0 = false;
-            if (bdx == 1) {
-                const int wb = g.Lx - x0;
-                if (wb <= 32 && ((mb >> wb) & 1ull)) {
-                    mb &= ~(1ull << wb);
-                    wrap0 = true;
-                }
-            }
-            if (BLOCKED) {
-                const uint32_t rowbytes = 4u * (uint32_t)g.RW;
-                const uint32_t ra = g.lat_addr + rowbytes * (uint32_t)lr;
-                const uint32_t rb = g.lat_addr + rowbytes * (uint32_t)(lr + bdy);
-                if (bdy == 0) {
-                    flip_row(g, ra, j, (unsigned long long)acc | mb, 0u, true);
-                } else {
-                    flip_row(g, ra, j, (unsigned long long)acc, 0u, true);
-                    flip_row(g, rb, j, mb, 0u, true);
-                }
-                if (wrap0) flip_row(g, rb, 0, 1ull, 0u, true);
-            } else {
-                const int yu = lr - g.D + g.Y0;  // unwrapped band row
-                if (bdy == 0) {
-                    flip_global_row(g, yu, j, (unsigned long long)acc | mb);
-                } else {
-                    flip_global_row(g, yu, j, (unsigned long long)acc);
-                    flip_global_row(g, yu + bdy, j, mb);
-                }
-                if (wrap0) flip_global_row(g, yu + bdy, 0, 1ull);
-            }
-        }
+        tl += NT;
+        if (tl < h.nlane) k = load_task<BLOCKED>(lat, g, tl, h.code >> 2, P, use_tab, tab);
     }
 }
 
@@ -336,7 +338,7 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
     Planes S = {0u, 0u, 0u};
     int ybase = 0, j = 0, lr = 0;
     if (valid) {
-        const int mi = (int)(((unsigned long long)t * g.magicW) >> 32);
+        const int mi = task_row(g, t);
         j = t - mi * g.W;
         if (use_tab) {
             const int2 r = tt->row[mi];
@@ -353,7 +355,7 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
             ybase = y * g.Lx;
             am = anchor_mask(j << 5, P, g.Lx);
         }
-        evaluate<G, OI>(lat + (size_t)lr * g.RW, g.RW, j, ta, tb, S);
+        evaluate<G, OI, true>(lat + lr * g.RW + j, g.RW, word_ends(j, g.W, g.nlast, 0), ta, tb, S);
     }
     const uint32_t unl = (ta ^ tb) & am;
     T.dmask = unl & draw_positions(S, g.sign);
@@ -372,54 +374,18 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
 template <int OI>
 __device__ __forceinline__ void band_task_finish(const Geo &g, const TaskPrep &T, uint32_t acc, Acc &A)
 {
-    constexpr int bdy = OI == 0 ? 0 : (OI == 1 ? 1 : -1);
-    constexpr int bdx = OI == 1 ? 0 : 1;
     if (!acc) return;
     if (T.own) {
         const int na = __popc(acc);
         A.acc += na;
-        A.dn += 2 * half_dn(T.S, acc, na);
+        A.dn += half_dn(T.S, acc, na);
     }
-    const int j = T.j, lr = T.lr, x0 = j << 5;
-    unsigned long long mb = (unsigned long long)acc << bdx;
-    bool wrap0 = false;
-    if (bdx == 1) {
-        const int wb = g.Lx - x0;
-        if (wb <= 32 && ((mb >> wb) & 1ull)) {
-            mb &= ~(1ull << wb);
-            wrap0 = true;
-        }
-    }
-    const uint32_t rowbytes = 4u * (uint32_t)g.RW;
-    if (j != 0 && 32 * j + 65 <= g.Lx) {
-        // a word clear of both row ends: no pad copies, no wrap, exact words
-        const uint32_t wa = g.lat_addr + rowbytes * (uint32_t)lr + 4u * (uint32_t)(j + 1);
-        const uint32_t wbw = wa + rowbytes * (uint32_t)bdy;
-        const uint32_t lo = (uint32_t)mb, hi = (uint32_t)(mb >> 32);
-        // every word is XORed, zero or not: an atomic of 0 costs less than a branch
-        if (bdy == 0) {
-            red_xor_local(wa, acc | lo);
-        } else {
-            red_xor_local(wa, acc);
-            red_xor_local(wbw, lo);
-        }
-        red_xor_local(wbw + 4u, hi);
-        return;
-    }
-    const uint32_t ra = g.lat_addr + rowbytes * (uint32_t)lr;
-    const uint32_t rb = g.lat_addr + rowbytes * (uint32_t)(lr + bdy);
-    if (bdy == 0) {
-        flip_row(g, ra, j, (unsigned long long)acc | mb, 0u, true);
-    } else {
-        flip_row(g, ra, j, (unsigned long long)acc, 0u, true);
-        flip_row(g, rb, j, mb, 0u, true);
-    }
-    if (wrap0) flip_row(g, rb, 0, 1ull, 0u, true);
+    flip_pairs<OI>(g.lat_addr + 4u * (uint32_t)(T.lr * g.RW + T.j), g.RW, word_ends(T.j, g.W, g.nlast, 0), acc);
 }
 
-template <int G, int OI, int THREADS, bool RK>
+template <int G, int OI, int THREADS>
 __device__ __forceinline__ void run_phase_pair(const uint32_t *lat, const Geo &g, const PhaseR &P,
-                                               const uint64_t *thr, int f, uint32_t s_lo, uint32_t s_hi,
+                                               const DrawThr &T, int f, uint32_t s_lo, uint32_t s_hi,
                                                Acc &A, uint32_t *q, const TaskTab *tt, const uint32_t (&rk)[2][8])
 {
     const int lane = threadIdx.x & 31;
@@ -432,30 +398,20 @@ __device__ __forceinline__ void run_phase_pair(const uint32_t *lat, const Geo &g
         band_task_prep<G, OI>(lat, g, P, use_tab, tt, ta, ta < ntask, T0, A);
         band_task_prep<G, OI>(lat, g, P, use_tab, tt, tb, tb < ntask, T1, A);
         uint32_t a0, a1;
-        draw_accepts_queue2<RK>(T0.dmask, T0.S, T0.base, T1.dmask, T1.S, T1.base, dk, rk, thr, q, a0, a1);
+        draw_accepts_queue2(T0.dmask, T0.S, T0.base, T1.dmask, T1.S, T1.base, dk, rk, T, q, a0, a1);
         band_task_finish<OI>(g, T0, T0.acc | a0, A);
         band_task_finish<OI>(g, T1, T1.acc | a1, A);
     }
 }
 
-template <int G, int THREADS, bool RK>
+template <int G, int THREADS>
 __device__ __forceinline__ void run_phase_pair_oi(const uint32_t *lat, const Geo &g, const PhaseR &P,
-                                                  const uint64_t *thr, int f, uint32_t s_lo, uint32_t s_hi,
+                                                  const DrawThr &T, int f, uint32_t s_lo, uint32_t s_hi,
                                                   Acc &A, uint32_t *q, const TaskTab *tt, const uint32_t (&rk)[2][8])
 {
-    if (P.oi == 0) run_phase_pair<G, 0, THREADS, RK>(lat, g, P, thr, f, s_lo, s_hi, A, q, tt, rk);
-    else if (G == kTRI6 && P.oi == 2) run_phase_pair<G, 2, THREADS, RK>(lat, g, P, thr, f, s_lo, s_hi, A, q, tt, rk);
-    else run_phase_pair<G, 1, THREADS, RK>(lat, g, P, thr, f, s_lo, s_hi, A, q, tt, rk);
-}
-
-template <int G, int THREADS, bool BLOCKED>
-__device__ __forceinline__ void run_phase_oi(const uint32_t *lat, const Geo &g, const PhaseR &P,
-                                             const uint64_t *thr, int f, uint32_t s_lo,
-                                             uint32_t s_hi, Acc &A, const TaskTab *tt = nullptr)
-{
-    if (P.oi == 0) run_phase<G, 0, THREADS, BLOCKED>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
-    else if (G == kTRI6 && P.oi == 2) run_phase<G, 2, THREADS, BLOCKED>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
-    else run_phase<G, 1, THREADS, BLOCKED>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
+    if (P.oi == 0) run_phase_pair<G, 0, THREADS>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
+    else if (G == kTRI6 && P.oi == 2) run_phase_pair<G, 2, THREADS>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
+    else run_phase_pair<G, 1, THREADS>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
 }
 
 template <typename T>
@@ -477,6 +433,13 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t v;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(v));
+    return v;
+}
+
+__device__ __forceinline__ uint32_t dynamic_smem_bytes()
+{
+    uint32_t v;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(v));
     return v;
 }
 
@@ -507,55 +470,140 @@ __host__ __device__ __forceinline__ int block_phases(int Lx, int Ly, int C)
 }
 
 // Phase table of (sweep s, phase f): the band's anchors, widened for a block.
-__device__ __forceinline__ void phase_table(const SweepJob &J, const Geo &g, int K, long long s, int f,
-                                            PhaseR *P)
+__device__ __forceinline__ void phase_table(const Geo &g, int K, long long s, int f, PhaseR *P)
 {
-    const int e = K > 1 ? 2 * (K - 1 - f % K) + 1 : 0;
-    phase_ranges(J.geometry, g.Lx, g.Ly, g.W, g.Y0 - e, g.Y1 + e, g.k0, g.k1, s, f, P);
+    const int e = K > 1 ? 2 * (K - 1 - (f & (K - 1))) + 1 : 0;
+    phase_ranges(g.tri ? kTRI6 : kSQ4, g.Lx, g.Ly, g.W, g.Y0 - e, g.Y1 + e, g.k0, g.k1, s, f, P);
 }
 
-// End of a block: the D lowest and D highest band rows go to the mailboxes of
-// parity p in the neighbouring CTAs, a cluster barrier, then this CTA's own
-// mailboxes of parity p fill its halo rows.
-template <int THREADS>
-__device__ __forceinline__ void exchange_halos(uint32_t *lat, const Geo &g, int hmax, int p)
+// Polls of a wait before it gives up; once one has, the launch's other waits poll once.
+constexpr int kExchangePolls = 1 << 20;
+
+// Waits for phase `parity` of the mbarrier at shared address bar, which the stores of
+// another CTA of the cluster complete.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int limit)
+{
+    for (int i = 0; i < limit; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// What a CTA's block exchanges need: its two mbarriers (side 0: from the CTA above,
+// side 1: from the one below) and the distances from its own shared memory to theirs.
+struct Exchange {
+    uint32_t bar, to_prev, to_next;
+    int polls;
+    bool fault;
+};
+
+// End of a block: the D lowest and D highest band rows go to the mailboxes of parity
+// block & 1 in the neighbouring CTAs, by asynchronous stores that count their bytes on
+// the receiver's mbarriers; this CTA's own mailboxes then fill its halo rows.  A CTA
+// waits for its two neighbours only.  Two parities are enough: a neighbour's block
+// n + 2 follows its receipt of this CTA's n + 1, sent after n was read; and the two
+// sides count apart, because one neighbour may be a block ahead of the other.
+// (With a cluster barrier instead, whose release waits for the stores to be
+// acknowledged, an exchange took about 0.8 us of a 400^2 lattice on 16 CTAs.)
+template <int NT>
+__device__ __forceinline__ void exchange_halos(uint32_t *lat, const Geo &g, int hmax, int block, Exchange &X)
 {
     const int H = g.Y1 - g.Y0, D = g.D, rw = D * g.RW;
-    uint32_t *mbox = lat + (size_t)(hmax + 2 * D) * g.RW;
-    const uint32_t prev = g.rank == 0 ? g.C - 1 : g.rank - 1;
-    const uint32_t next = g.rank + 1 == g.C ? 0 : g.rank + 1;
-    for (int idx = threadIdx.x; idx < 2 * rw; idx += THREADS) {
-        const int side = idx >= rw ? 1 : 0;
-        const int k = idx - side * rw;
-        const uint32_t v = lat[(size_t)(side ? D : H) * g.RW + k];
-        const uint32_t local = smem_addr(mbox + (size_t)(2 * p + side) * rw + k);
-        uint32_t remote;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                     : "=r"(remote) : "r"(local), "r"(side ? prev : next));
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+    const uint32_t p = (uint32_t)block & 1u;
+    uint32_t *const mbox = lat + (hmax + 2 * D) * g.RW + 2 * p * rw;
+    const uint32_t mbox_addr = g.lat_addr + 4u * (uint32_t)((hmax + 2 * D) * g.RW + 2 * p * rw);
+    if (threadIdx.x < 2) {
+        unsigned long long st;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;"
+                     : "=l"(st) : "r"(X.bar + 8u * threadIdx.x), "r"(4u * (uint32_t)rw) : "memory");
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    for (int idx = threadIdx.x; idx < 2 * rw; idx += THREADS) {
-        const int side = idx >= rw ? 1 : 0;
-        const int k = idx - side * rw;
-        lat[(size_t)(side ? D + H : 0) * g.RW + k] = mbox[(size_t)(2 * p + side) * rw + k];
+    for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
+        const bool low = idx >= rw;  // the lowest rows go up (side 1 there), the highest down (side 0)
+        const uint32_t v = lat[low ? D * g.RW + idx - rw : H * g.RW + idx];
+        const uint32_t to = low ? X.to_prev : X.to_next;
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                     ::"r"(mbox_addr + 4u * (uint32_t)idx + to), "r"(v), "r"(X.bar + (low ? 8u : 0u) + to) : "memory");
     }
-    __syncthreads();
+    for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
+        const bool low = idx >= rw;
+        if (!mbar_wait_cluster(X.bar + (low ? 8u : 0u), p, X.polls)) {
+            X.polls = 1;
+            X.fault = true;
+        }
+        lat[low ? (D + H) * g.RW + idx - rw : idx] = mbox[idx];
+    }
 }
 
+// Distance from a shared address of this CTA to the same one of CTA `rank`.
+__device__ __forceinline__ uint32_t mapa_distance(uint32_t addr, int rank)
+{
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    return remote - addr;
+}
+
+// Words of the task tables of one phase, and of the two chunks' (see TaskTab): anchor
+// masks of W words (even, so that the row entries stay aligned) and the rows.
+__host__ __device__ __forceinline__ int phase_table_words(int W, int hmax, int K)
+{
+    return ((W + 1) & ~1) + 2 * ((hmax + 4 * K) / 2 + 2);  // anchor rows of hmax + 2(2K - 1) rows, 2 apart
+}
+__host__ __device__ __forceinline__ long long chunk_table_words(int W, int hmax, int K)
+{
+    return 2ll * kChunk * phase_table_words(W, hmax, K);
+}
+// Words of a CTA's rows (and mailboxes), where the tables start.
+__host__ __device__ __forceinline__ long long resident_row_words(int RW, int hmax, int K)
+{
+    return ((long long)RW * (K > 1 ? hmax + 6 * (2 * K + 1) : hmax + 4) + 1) & ~1ll;
+}
+
+// Schedule entry and draw key of phase f of sweep s.
+template <int NT>
+__device__ __forceinline__ void prepare_entry(const Geo &g, int K, long long s, int f, PhaseR *P,
+                                              PhaseHdr *h)
+{
+    phase_table(g, K, s, f, P);
+    const DrawKey dk = draw_key((uint32_t)f, (uint32_t)(unsigned long long)s, (uint32_t)((unsigned long long)s >> 32),
+                                g.k0, g.k1);
+    const int ls = word_split<NT>(P->ntask);
+    h->nlane = P->ntask << ls;
+    h->code = P->oi + 4 * ls;
+    h->hk = dk.hk;
+    h->la = dk.la;
+}
+
+template <int V>
+using Const = std::integral_constant<int, V>;
+
+// Preparing a phase (a Philox block, the anchor rows' ranges, the tables) takes one
+// warp about 1100 cycles, as long as a phase of a lattice spread over a cluster.  So
+// with more than 128 threads the last kAhead warps do nothing else: they prepare the
+// next kChunk phases while the others, which synchronise among themselves, run the
+// current ones, and meet them once per chunk.  With 128 threads (several CTAs per SM,
+// every warp busy) each of the four warps prepares one phase of the next chunk before
+// its own tasks.
 template <int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB)
 resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__restrict__ calls,
                       const int *__restrict__ job_map, const SweepJob job0, const SweepCall call0)
 {
     constexpr int kWarps = THREADS / 32;
+    constexpr int kAhead = THREADS > 256 ? 4 : (THREADS > 128 ? 2 : 0);
+    constexpr int NT = THREADS - 32 * kAhead;  // threads with tasks
+    constexpr int kPrep = kAhead > 0 ? kAhead : kWarps;  // warps that prepare
+    static_assert(kPrep <= kChunk && kChunk % kPrep == 0, "each preparing warp has kChunk / kPrep phases");
     extern __shared__ __align__(16) uint32_t lat[];
-    __shared__ PhaseR pp[2][8];
-    __shared__ uint64_t thr[kThrEntries];
+    __shared__ PhaseR pp[2][kChunk];
+    __shared__ PhaseHdr hdr[2][kChunk];
     __shared__ long long red[5][kWarps];
-    __shared__ uint32_t tab_am[2][kTabW];   // tables of the current and the next phase
-    __shared__ int2 tab_row[2][kTabRows];
+    __shared__ __align__(8) unsigned long long xbar[2];
 
     const int C = (int)cluster_nctarank();
     const int rank = (int)cluster_ctarank();
@@ -565,10 +613,12 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     if (Cl.n_mcs <= 0) return;  // uniform over the cluster
 
     Geo g;
-    g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = J.RW; g.magicW = J.magicW;
+    g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = J.RW; g.magicW = g.W == 1 ? 0u : (uint32_t)J.magicW; g.one = g.W == 1 ? ~0u : 0u;
+    g.nlast = g.Lx - 32 * (g.W - 1);
     g.k0 = J.key0; g.k1 = J.key1;
     // The host's draw range is [z, 2(z-1)] (omega > 0), [0, z-2] (omega < 0) or empty.
     g.sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
+    g.tri = J.geometry == kTRI6;
     g.C = C;
     g.rank = rank;
     g.Y0 = (int)(((long long)rank * g.Ly) / C);
@@ -596,112 +646,156 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         int y = g.Y0 - g.D + lr;
         y %= g.Ly;
         if (y < 0) y += g.Ly;
-        lat[idx] = padded_word(J.lat, J.packing, J.pitch, y, w, g.Lx, g.W);
+        lat[idx] = w < g.W ? store_word(J.lat, J.packing, J.pitch, y, w, g.Lx) : 0u;
     }
-    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
-    // The last three warps prepare the next phase while the phase runs: its anchor
-    // masks, its rows, and (lane 0) one schedule entry of the next sweep.
-    const int warp = tid >> 5;
-    const bool table_warp = warp == kWarps - 1;
-    const bool row_warp = warp == kWarps - 2;
-    const bool sched_warp = warp == kWarps - 3;
-    if (table_warp) {
-        if ((tid & 31) < 8) phase_table(J, g, K, Cl.sweep0, tid & 31, &pp[0][tid & 31]);
+    // The tables follow the rows where the launch's shared memory holds them.
+    const int tab_words = phase_table_words(g.W, hmax, K);
+    uint32_t *const tab_base = lat + resident_row_words(g.RW, hmax, K);
+    const bool tables = 4 * (resident_row_words(g.RW, hmax, K) + chunk_table_words(g.W, hmax, K)) <=
+                        (long long)dynamic_smem_bytes();
+    const int warp = tid >> 5, lane = tid & 31;
+    const bool ahead_warp = kAhead > 0 && warp >= kWarps - kAhead;
+    const DrawThr T = draw_thresholds(J);
+    g.tabW = (g.W + 1) & ~1;
+    unsigned long long t_att = 0, t_unl = 0, t_drw = 0, t_acc = 0;
+    long long t_dn = 0;
+    // Prepares chunk c (sweep c / 2, its phases kChunk (c & 1) ..) into buffer c & 1.
+    auto prepare_chunk = [&](long long c) {
+        const int buf = (int)(c & 1), f0 = kChunk * buf;
+        const long long s = Cl.sweep0 + (c >> 1);
+        if (kAhead > 0 && !ahead_warp) return;
+        constexpr int kPer = kChunk / kPrep;
+        const int q0 = (warp - (kWarps - kPrep)) * kPer;
+        if (lane < kPer) {
+            PhaseR *const P = &pp[buf][q0 + lane];
+            prepare_entry<NT>(g, K, s, f0 + q0 + lane, P, &hdr[buf][q0 + lane]);
+            if (rank == 0) t_att += (unsigned long long)P->att;  // the whole lattice's, counted once
+        }
         __syncwarp();
-        const TaskTab T0 = {tab_am[0], tab_row[0], kTabW, kTabRows};
-        if (blocked) build_task_table<true>(pp[0][0], g, T0, tid & 31, 32);
-        else build_task_table<false>(pp[0][0], g, T0, tid & 31, 32);
-    }
+        if (!tables) return;
+#pragma unroll 1
+        for (int q = q0; q < q0 + kPer; ++q) {
+            const PhaseR P = pp[buf][q];
+            uint32_t *const t = tab_base + (buf * kChunk + q) * tab_words;
+            const TaskTab tt = {t, (int2 *)(t + g.tabW), g.W, tab_words};
+            if (blocked) build_task_table<true>(P, g, tt, lane, 32);
+            else build_task_table<false>(P, g, tt, lane, 32);
+        }
+    };
+    prepare_chunk(0);
+    if (tid < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&xbar[tid])) : "memory");
+    if (tid < 2) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // Every CTA of the cluster must be running before any peer writes into it.
-    if (C > 1) {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    } else {
-        __syncthreads();
-    }
+    if (C > 1) cluster_barrier();
+    else cta_barrier();
 
     // Start energy for the trace, read before any CTA of this lattice can finish.
     const long long n_unlike0 = (tid == 0 && rank == 0 && Cl.trace_every > 0) ? J.state[kNUnlike] : 0;
-    unsigned long long t_att = 0, t_unl = 0, t_drw = 0, t_acc = 0;
-    long long t_dn = 0;
-    int block = 0;
-    for (long long it = 0; it < Cl.n_mcs; ++it) {
-        const long long s = Cl.sweep0 + it;
-        const uint32_t s_lo = (uint32_t)(unsigned long long)s;
-        const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
-        const int buf = (int)(it & 1);
-        Acc A = {0u, 0u, 0u, 0};
-        for (int f = 0; f < 8; ++f) {
-            const bool last = f == 7 && it + 1 == Cl.n_mcs;
-            if ((table_warp || row_warp) && !last) {
-                // the next phase's task table (phase 0 of the next sweep after phase 7)
-                const PhaseR Pn = f == 7 ? pp[buf ^ 1][0] : pp[buf][f + 1];
-                const TaskTab Tn = {tab_am[(f + 1) & 1], tab_row[(f + 1) & 1], kTabW, kTabRows};
-                if (table_warp) {
-                    if (blocked) build_task_table<true, true, false>(Pn, g, Tn, tid & 31, 32);
-                    else build_task_table<false, true, false>(Pn, g, Tn, tid & 31, 32);
-                } else {
-                    if (blocked) build_task_table<true, false, true>(Pn, g, Tn, tid & 31, 32);
-                    else build_task_table<false, false, true>(Pn, g, Tn, tid & 31, 32);
+    // The preparing warps: the next chunk's tables while the current one runs, then the
+    // chunk's last barrier (every phase is a cluster barrier when bands are too thin
+    // for blocks).
+    Exchange X = {smem_addr(&xbar[0]), 0u, 0u, kExchangePolls, false};
+    auto run_tasks = [&](auto geometry, auto is_blocked, auto has_fix) {
+        constexpr int G = decltype(geometry)::value;
+        constexpr bool BLOCKED = decltype(is_blocked)::value, FIX = decltype(has_fix)::value;
+        int block = 0;
+        for (long long it = 0; it < Cl.n_mcs; ++it) {
+            const bool last = it + 1 == Cl.n_mcs;
+            const long long s = Cl.sweep0 + it;
+            DrawKey dk = draw_key(0u, (uint32_t)(unsigned long long)s, (uint32_t)((unsigned long long)s >> 32), g.k0,
+                                  g.k1);
+            Acc A = {0u, 0u, 0u, 0};
+#pragma unroll 1
+            for (int buf = 0; buf < 8 / kChunk; ++buf) {
+                if (kAhead == 0 && !(last && buf == 1)) prepare_chunk(2 * it + buf + 1);
+                const PhaseHdr *hp = hdr[buf];
+                const uint32_t *tab = tab_base + buf * kChunk * tab_words;
+                PhaseHdr h = hp[0];
+                Task k = {};
+                if (tid < h.nlane) k = load_task<BLOCKED>(lat, g, tid, h.code >> 2, pp[buf][0], tables, tab);
+#pragma unroll 1
+                for (int q = 0; q < kChunk; ++q) {
+                    dk.hk = h.hk;
+                    dk.la = h.la;
+                    const int oi = h.code & 3;
+                    const PhaseR &P = pp[buf][q];
+                    if (oi == 0) run_phase<G, 0, NT, BLOCKED, FIX>(lat, g, h, k, P, T, dk, A, tables, tab);
+                    else if (G == kSQ4 || oi == 1) run_phase<G, 1, NT, BLOCKED, FIX>(lat, g, h, k, P, T, dk, A, tables, tab);
+                    else run_phase<G, 2, NT, BLOCKED, FIX>(lat, g, h, k, P, T, dk, A, tables, tab);
+                    if (q < kChunk - 1) {  // the next phase's entry does not wait for this one
+                        tab += tab_words;
+                        h = hp[q + 1];
+                        if (tid < h.nlane) k = load_task<BLOCKED>(lat, g, tid, h.code >> 2, pp[buf][q + 1], tables, tab);
+                    }
+                    if (!BLOCKED && C > 1) {
+                        cluster_barrier();
+                        continue;
+                    }
+                    // Blocks of K phases end with an exchange, except the launch's last.
+                    if (BLOCKED && ((q + 1) & (K - 1)) == 0 && !(last && buf == 1 && q == kChunk - 1)) {
+                        task_barrier<NT>();
+                        exchange_halos<NT>(lat, g, hmax, block++, X);
+                    }
+                    if (q == kChunk - 1) cta_barrier();
+                    else task_barrier<NT>();
                 }
             }
-            // Phase f of the next sweep: one schedule entry per phase.  (Entry f of the
-            // other buffer was last read in phase f of the previous sweep; phase 0's is
-            // written here before phase 7 builds its task table from it.)
-            if (sched_warp && (tid & 31) == 0) {
-                if (it + 1 < Cl.n_mcs) phase_table(J, g, K, s + 1, f, &pp[buf ^ 1][f]);
-                if (rank == 0) t_att += (unsigned long long)pp[buf][f].att;  // the lattice's, counted once
+            t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
+            t_dn += 2 * A.dn;
+            // Energy trace: each CTA adds its cumulative dn; CTA 0 adds the start value
+            // (the launcher zeroes the trace buffer).
+            if (Cl.trace_every > 0 && (it + 1) % Cl.trace_every == 0) {
+                const long long ws = warp_sum(t_dn);
+                if (lane == 0 && ws != 0)
+                    atomicAdd((unsigned long long *)&Cl.trace[(it + 1) / Cl.trace_every - 1],
+                              (unsigned long long)ws);
+                if (tid == 0 && rank == 0)
+                    atomicAdd((unsigned long long *)&Cl.trace[(it + 1) / Cl.trace_every - 1],
+                              (unsigned long long)n_unlike0);
             }
-            const PhaseR P = pp[buf][f];
-            const TaskTab Tc = {tab_am[f & 1], tab_row[f & 1], kTabW, kTabRows};
-            const TaskTab *tt = &Tc;
-            if (blocked) {
-                if (J.geometry == kTRI6)
-                    run_phase_oi<kTRI6, THREADS, true>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
-                else
-                    run_phase_oi<kSQ4, THREADS, true>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
-                __syncthreads();
-                if (f % K == K - 1 && !(f == 7 && it + 1 == Cl.n_mcs)) {
-                    exchange_halos<THREADS>(lat, g, hmax, block & 1);
-                    ++block;
-                }
+        }
+    };
+    if (ahead_warp) {
+        for (long long c = 1; c <= 2 * Cl.n_mcs; ++c) {
+            if (c < 2 * Cl.n_mcs) prepare_chunk(c);
+            if (blocked || C == 1) {
+                cta_barrier();
             } else {
-                if (J.geometry == kTRI6)
-                    run_phase_oi<kTRI6, THREADS, false>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
-                else
-                    run_phase_oi<kSQ4, THREADS, false>(lat, g, P, thr, f, s_lo, s_hi, A, tt);
-                phase_barrier(C);
+                for (int q = 0; q < kChunk; ++q) cluster_barrier();
             }
         }
-        t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
-        t_dn += A.dn;
-        // Energy trace: each CTA adds its cumulative dn; CTA 0 adds the start value
-        // (the launcher zeroes the trace buffer).
-        if (Cl.trace_every > 0 && (it + 1) % Cl.trace_every == 0) {
-            const long long ws = warp_sum(t_dn);
-            if ((tid & 31) == 0 && ws != 0)
-                atomicAdd((unsigned long long *)&Cl.trace[(it + 1) / Cl.trace_every - 1],
-                          (unsigned long long)ws);
-            if (tid == 0 && rank == 0)
-                atomicAdd((unsigned long long *)&Cl.trace[(it + 1) / Cl.trace_every - 1],
-                          (unsigned long long)n_unlike0);
+    } else if (blocked) {
+        X.to_prev = mapa_distance(g.lat_addr, rank == 0 ? C - 1 : rank - 1);
+        X.to_next = mapa_distance(g.lat_addr, rank + 1 == C ? 0 : rank + 1);
+        // (rows whose last word holds one site take a longer window: their own copy)
+        if (g.nlast == 1) {
+            if (g.tri) run_tasks(Const<kTRI6>{}, std::true_type{}, std::true_type{});
+            else run_tasks(Const<kSQ4>{}, std::true_type{}, std::true_type{});
+        } else {
+            if (g.tri) run_tasks(Const<kTRI6>{}, std::true_type{}, std::false_type{});
+            else run_tasks(Const<kSQ4>{}, std::true_type{}, std::false_type{});
         }
+    } else {
+        if (g.tri) run_tasks(Const<kTRI6>{}, std::false_type{}, std::true_type{});
+        else run_tasks(Const<kSQ4>{}, std::false_type{}, std::true_type{});
+    }
+    // A wait that ran out leaves a lattice that is no state of the chain: report it, and
+    // give stores in flight a second bounded wait.  No CTA leaves while a peer may still
+    // write into it.
+    if (blocked) {
+        if (__syncthreads_or(X.fault)) {
+            if (tid == 0) atomicExch((unsigned long long *)&J.state[kFault], 1ull);
+            for (int side = 0; side < 2; ++side)
+                for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * side, par, kExchangePolls);
+        }
+        cluster_barrier();
     }
 
     // Write the band back (main positions only).
     for (int idx = tid; idx < H * g.W; idx += THREADS) {
         const int r = idx / g.W, w = idx - r * g.W;
         const int y = g.Y0 + r;
-        const uint32_t v = lat[(size_t)(r + g.D) * g.RW + w + 1];
-        const int pos0 = 32 * w;
-        const int nvalid = min(32, g.Lx - pos0);
-        if (J.packing == kPackBit) {
-            const uint32_t valid = nvalid == 32 ? 0xFFFFFFFFu : ((1u << nvalid) - 1u);
-            ((uint32_t *)J.lat)[(size_t)y * J.pitch + w] = v & valid;
-        } else {
-            uint8_t *row = (uint8_t *)J.lat + (size_t)y * J.pitch;
-            for (int b = 0; b < nvalid; ++b) row[pos0 + b] = (uint8_t)((v >> b) & 1u);
-        }
+        write_word(J.lat, J.packing, J.pitch, y, w, g.Lx, lat[(r + g.D) * g.RW + w]);
     }
 
     // Counters and energy.
@@ -782,22 +876,23 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     constexpr int kWarps = THREADS / 32;
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ PhaseR pp[8];
-    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
     __shared__ __align__(8) unsigned long long copy_bar;
     // The next launch may be scheduled now; it waits for this one before it reads.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     Geo g;
-    g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = band_row_words(J.W); g.magicW = J.magicW;
+    g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = band_row_words(J.W); g.magicW = g.W == 1 ? 0u : (uint32_t)J.magicW; g.one = g.W == 1 ? ~0u : 0u;
+    g.nlast = g.Lx - 32 * (g.W - 1);
     g.k0 = J.key0; g.k1 = J.key1;
     g.sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
+    g.tri = J.geometry == kTRI6;
     g.C = (int)gridDim.x;
     g.rank = (int)blockIdx.x;
     g.Y0 = (int)blockIdx.x * H;
     g.Y1 = min(g.Y0 + H, g.Ly);
     g.prevY = g.prevH = g.nextY = g.nextH = 0;
-    uint32_t *const lat = smem + 3;  // padded row lr, word w: lat[lr * RWb + w]
+    uint32_t *const lat = smem;
     g.lat_addr = smem_addr(lat);
     g.D = 2 * K + 1;
     g.base = g.Y0 - g.D < 0 ? g.Y0 - g.D + g.Ly : g.Y0 - g.D;
@@ -816,11 +911,10 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     }
     // Everything below reads what earlier launches on the stream wrote.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
     const long long s = J.state[kSweepBase] + k;
     const uint32_t s_lo = (uint32_t)(unsigned long long)s;
     const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
-    if (tid < K) phase_table(J, g, K, s, f0 + tid, &pp[tid]);
+    if (tid < K) phase_table(g, K, s, f0 + tid, &pp[tid]);
 
     if (bulk) {
         // One bulk copy per row (pitch words, 16-byte aligned at both ends) into the
@@ -844,7 +938,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
                 if (y < 0) y += g.Ly;
                 if (y >= g.Ly) y -= g.Ly;
                 const char *from = (const char *)src + (size_t)y * row_bytes;
-                const uint32_t to = smem_addr(lat + (size_t)lr * RWb + 1);
+                const uint32_t to = smem_addr(lat + (size_t)lr * RWb);
                 asm volatile(
                     "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                     ::"r"(to), "l"(from), "r"(row_bytes), "r"(bar) : "memory");
@@ -860,26 +954,13 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
             mbar_wait(bar, 0u, polls);
             return;
         }
-        for (int lr = tid; lr < NL; lr += THREADS) {
-            uint32_t *row = lat + (size_t)lr * RWb;
-            const int xl = g.Lx - 1;
-            const uint32_t s01 = row[1] & 3u;
-            const uint32_t last = (row[(xl >> 5) + 1] >> (xl & 31)) & 1u;
-            const int nvalid = g.Lx - 32 * (g.W - 1);
-            if (nvalid < 32) row[g.W] &= (1u << nvalid) - 1u;
-            for (int w = g.W + 1; w <= J.pitch; ++w) row[w] = 0u;  // beyond the sites
-            row[g.W + 1] = 0u;
-            row[(g.Lx + 32) >> 5] |= (s01 & 1u) << (g.Lx & 31);       // position Lx: site 0
-            row[(g.Lx + 33) >> 5] |= (s01 >> 1) << ((g.Lx + 1) & 31);  // position Lx + 1: site 1
-            row[0] = last << 31;                                         // position -1: site Lx - 1
-        }
     } else {
-        for (int idx = tid; idx < NL * (g.W + 2); idx += THREADS) {
-            const int lr = idx / (g.W + 2), w = idx - lr * (g.W + 2);
+        for (int idx = tid; idx < NL * g.W; idx += THREADS) {
+            const int lr = idx / g.W, w = idx - lr * g.W;
             int y = g.Y0 - g.D + lr;
             if (y < 0) y += g.Ly;
             if (y >= g.Ly) y -= g.Ly;
-            lat[(size_t)lr * RWb + w] = padded_word(src, J.packing, J.pitch, y, w, g.Lx, g.W);
+            lat[(size_t)lr * RWb + w] = store_word(src, J.packing, J.pitch, y, w, g.Lx);
         }
     }
     __syncthreads();
@@ -897,6 +978,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     }
 
     Acc A = {0u, 0u, 0u, 0};
+    const DrawThr DT = draw_thresholds(J);
     // the warps' draw queues follow the rows (H + 2D rows of the tallest band)
     uint32_t *const dq = smem + (size_t)(H + 2 * g.D) * RWb + (size_t)(tid >> 5) * kDrawQueue2Words;
     dq[kDrawQueue2Acc + (tid & 31)] = 0u;  // the queue's accept words start at zero
@@ -907,26 +989,20 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
         const TaskTab T = {t, (int2 *)(t + tab_w), g.W, tab_rows};
         const TaskTab *const tt = tables ? &T : nullptr;
         if (J.geometry == kTRI6)
-            run_phase_pair_oi<kTRI6, THREADS, true>(lat, g, P, thr, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+            run_phase_pair_oi<kTRI6, THREADS>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
         else
-            run_phase_pair_oi<kSQ4, THREADS, true>(lat, g, P, thr, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+            run_phase_pair_oi<kSQ4, THREADS>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
         __syncthreads();
     }
 
     if (bulk) {
-        // The band's rows as stored: sites only, then one bulk copy per row.
-        for (int r = tid; r < Hc; r += THREADS) {
-            uint32_t *row = lat + (size_t)(r + g.D) * RWb;
-            const int nvalid = g.Lx - 32 * (g.W - 1);
-            if (nvalid < 32) row[g.W] &= (1u << nvalid) - 1u;
-            for (int w = g.W + 1; w <= J.pitch; ++w) row[w] = 0u;
-        }
+        // One bulk copy per row: flips left the words and bits past its end as they were read.
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (tid < 32) {
             for (int r = tid; r < Hc; r += 32) {
                 char *to = (char *)dst + (size_t)(g.Y0 + r) * row_bytes;
-                const uint32_t from = smem_addr(lat + (size_t)(r + g.D) * RWb + 1);
+                const uint32_t from = smem_addr(lat + (size_t)(r + g.D) * RWb);
                 asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                              ::"l"(to), "r"(from), "r"(row_bytes) : "memory");
             }
@@ -937,16 +1013,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
         for (int idx = tid; idx < Hc * g.W; idx += THREADS) {
             const int r = idx / g.W, w = idx - r * g.W;
             const int y = g.Y0 + r;
-            const uint32_t v = lat[(size_t)(r + g.D) * RWb + w + 1];
-            const int pos0 = 32 * w;
-            const int nvalid = min(32, g.Lx - pos0);
-            if (J.packing == kPackBit) {
-                const uint32_t valid = nvalid == 32 ? 0xFFFFFFFFu : ((1u << nvalid) - 1u);
-                ((uint32_t *)dst)[(size_t)y * J.pitch + w] = v & valid;
-            } else {
-                uint8_t *row = (uint8_t *)dst + (size_t)y * J.pitch;
-                for (int b = 0; b < nvalid; ++b) row[pos0 + b] = (uint8_t)((v >> b) & 1u);
-            }
+            write_word(dst, J.packing, J.pitch, y, w, g.Lx, lat[(size_t)(r + g.D) * RWb + w]);
         }
     }
 
@@ -954,7 +1021,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     if (blockIdx.x == 0 && tid == 0)
         for (int j = 0; j < K; ++j) att += pp[j].att;  // the whole lattice's, counted once
     long long vals[5] = {att, (long long)A.unl, (long long)A.drw, (long long)A.acc,
-                         (long long)A.dn};
+                         2ll * A.dn};
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
         const long long ws = warp_sum(vals[q]);
@@ -1040,11 +1107,29 @@ size_t resident_smem_bytes(int Lx, int Ly, int cluster)
     return RW * (H + 4) * sizeof(uint32_t);
 }
 
+size_t resident_launch_bytes(int Lx, int Ly, int cluster)
+{
+    const int C = cluster < 1 ? 1 : cluster;
+    const int K = block_phases(Lx, Ly, C), hmax = (Ly + C - 1) / C, W = (Lx + 31) / 32;
+    const size_t rows = resident_smem_bytes(Lx, Ly, C);
+    const size_t all = (size_t)(4 * (resident_row_words(W + 2, hmax, K) + chunk_table_words(W, hmax, K)));
+    return all <= (size_t)kResidentMaxSmem ? all : rows;
+}
+
 int resident_max_smem_bytes() { return kResidentMaxSmem; }
 
 int resident_block_phases(int Lx, int Ly, int cluster) { return block_phases(Lx, Ly, cluster); }
 
-int resident_default_threads(int cluster) { return cluster == 1 ? 512 : 256; }
+// A phase of a lattice spread over a cluster lasts as long as its busiest warp, so the
+// CTA has enough threads for one task each: 192 of 256 or 384 of 512 run tasks (the
+// others prepare).  GB300, us per phase at 256 / 512 threads: 64^2 on 4 CTAs 0.76 /
+// 0.81, 300^2 on 16 1.04 / 1.07, 350^2 1.18 / 1.12, 400^2 1.41 / 1.19.
+int resident_default_threads(int Lx, int Ly, int cluster)
+{
+    const int C = cluster < 1 ? 1 : cluster, K = block_phases(Lx, Ly, C);
+    const int rows = (Ly + C - 1) / C + (K > 1 ? 2 * (2 * K - 1) : 0);
+    return (long long)((rows + 1) / 2) * ((Lx + 31) / 32) > 192 ? 512 : 256;
+}
 
 int resident_max_cluster(int Ly)
 {

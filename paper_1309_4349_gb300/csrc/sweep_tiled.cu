@@ -2,8 +2,8 @@
 // memory: one kernel launch per phase over the device store.
 //
 // The grid splits the lattice into row bands of H rows, one CTA each.  A CTA stages
-// its band plus two halo rows on each side into shared memory (the padded row
-// layout of sweep_common.cuh), evaluates the phase's anchors of its band with the
+// its band plus two halo rows on each side into shared memory (the rows of
+// sweep_common.cuh), evaluates the phase's anchors of its band with the
 // same bit-sliced code as the resident kernel, draws, and applies accepted
 // exchanges to the device store with atomic XORs.  Within a phase no site of one
 // pair neighbours a site of another (the schedule is conflict-free), so no bit a
@@ -30,33 +30,27 @@ struct Acc {
     int32_t dn;
 };
 
-// XOR the sites x0 + i (bit i of m, x0 = 32 j, every site < Lx) of row y in the store.
-__device__ __forceinline__ void flip_store(const SweepJob &J, int y, int j, unsigned long long m)
+// XORs m into word j of row y of the store.
+__device__ __forceinline__ void flip_store(const SweepJob &J, int y, int j, uint32_t m)
 {
     if (J.packing == kPackBit) {
-        uint32_t *row = (uint32_t *)J.lat + (size_t)y * J.pitch;
-        const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32);
-        if (lo) atomicXor(row + j, lo);
-        if (hi) atomicXor(row + j + 1, hi);
+        if (m) atomicXor((uint32_t *)J.lat + (size_t)y * J.pitch + j, m);
         return;
     }
-    uint8_t *row = (uint8_t *)J.lat + (size_t)y * J.pitch;
+    uint32_t *const row = (uint32_t *)((uint8_t *)J.lat + (size_t)y * J.pitch + 32 * j);
     while (m) {
-        const int i = __ffsll((long long)m) - 1;
-        m &= m - 1ull;
-        const size_t off = (size_t)(row - (uint8_t *)J.lat) + (size_t)(32 * j + i);
-        uint32_t *word = (uint32_t *)((uint8_t *)J.lat + (off & ~(size_t)3));
-        atomicXor(word, 1u << (8 * (off & 3)));
+        const int i = __ffs(m) - 1;
+        m &= m - 1u;
+        atomicXor(row + (i >> 2), 1u << (8 * (i & 3)));
     }
 }
 
 template <int G, int OI>
 __device__ __forceinline__ void run_tiles(const uint32_t *tile, const SweepJob &J, const PhaseP &P,
-                                          int Y0, int sign, const uint64_t *thr, int f,
+                                          int Y0, int sign, const DrawThr &T, int f,
                                           uint32_t s_lo, uint32_t s_hi, Acc &A)
 {
     constexpr int bdy = OI == 0 ? 0 : (OI == 1 ? 1 : -1);
-    constexpr int bdx = OI == 1 ? 0 : 1;
     const DrawKey dk = draw_key((uint32_t)f, s_lo, s_hi, J.key0, J.key1);
     for (int t = threadIdx.x; t < P.ntask; t += kThreads) {
         const int mi = (int)(((unsigned long long)t * J.magicW) >> 32);
@@ -69,36 +63,26 @@ __device__ __forceinline__ void run_tiles(const uint32_t *tile, const SweepJob &
         if (am == 0u) continue;
         uint32_t ta, tb;
         Planes S;
-        evaluate<G, OI>(tile + (size_t)(y - Y0 + 2) * J.RW, J.RW, j, ta, tb, S);
+        const WordEnds E = word_ends(j, J.W, J.Lx - 32 * (J.W - 1), 0);
+        evaluate<G, OI, true>(tile + (size_t)(y - Y0 + 2) * J.RW + j, J.RW, E, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
         const uint32_t dmask = unl & draw_positions(S, sign);
         uint32_t acc = unl & ~dmask;
-        acc |= draw_accepts(dmask, S, (uint32_t)(y * J.Lx + x0), dk, thr);
+        acc |= draw_accepts(dmask, S, (uint32_t)(y * J.Lx + x0), dk, T);
         A.unl += __popc(unl);
         A.drw += __popc(dmask);
         if (acc) {
             const int na = __popc(acc);
             A.acc += na;
             A.dn += 2 * half_dn(S, acc, na);
-            unsigned long long mb = (unsigned long long)acc << bdx;
-            bool wrap0 = false;  // the pair of anchor Lx-1 wraps to site 0
-            if (bdx == 1) {
-                const int wb = J.Lx - x0;
-                if (wb <= 32 && ((mb >> wb) & 1ull)) {
-                    mb &= ~(1ull << wb);
-                    wrap0 = true;
-                }
-            }
+            uint32_t b;
+            const uint32_t next = partners<OI>(acc, E, b);
             int yb = y + bdy;
             if (yb < 0) yb += J.Ly;
             if (yb >= J.Ly) yb -= J.Ly;
-            if (bdy == 0) {
-                flip_store(J, y, j, (unsigned long long)acc | mb);
-            } else {
-                flip_store(J, y, j, (unsigned long long)acc);
-                flip_store(J, yb, j, mb);
-            }
-            if (wrap0) flip_store(J, yb, 0, 1ull);
+            flip_store(J, y, j, OI == 0 ? acc | b : acc);
+            if (OI != 0) flip_store(J, yb, j, b);
+            flip_store(J, yb, j + E.r, next);
         }
     }
 }
@@ -116,7 +100,6 @@ tiled_phase_kernel(const SweepJob J, int H, int k, int f)
 {
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ PhaseP P;
-    __shared__ uint64_t thr[kThrEntries];
     __shared__ long long red[5][kWarps];
 
     const int tid = threadIdx.x;
@@ -129,23 +112,23 @@ tiled_phase_kernel(const SweepJob J, int H, int k, int f)
         int y = Y0 - 2 + lr;
         if (y < 0) y += J.Ly;
         if (y >= J.Ly) y -= J.Ly;
-        tile[idx] = padded_word(J.lat, J.packing, J.pitch, y, w, J.Lx, J.W);
+        tile[idx] = w < J.W ? store_word(J.lat, J.packing, J.pitch, y, w, J.Lx) : 0u;
     }
     if (tid == 0) phase_params(J.geometry, J.Lx, J.Ly, J.W, Y0, Y1, J.key0, J.key1, s, f, &P);
-    if (tid < kThrEntries) thr[tid] = pair_threshold(J, tid);
     __syncthreads();
 
     const int sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
     const uint32_t s_lo = (uint32_t)(unsigned long long)s;
     const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
+    const DrawThr T = draw_thresholds(J);
     Acc A = {0u, 0u, 0u, 0};
     if (J.geometry == kTRI6) {
-        if (P.oi == 0) run_tiles<kTRI6, 0>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
-        else if (P.oi == 1) run_tiles<kTRI6, 1>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
-        else run_tiles<kTRI6, 2>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
+        if (P.oi == 0) run_tiles<kTRI6, 0>(tile, J, P, Y0, sign, T, f, s_lo, s_hi, A);
+        else if (P.oi == 1) run_tiles<kTRI6, 1>(tile, J, P, Y0, sign, T, f, s_lo, s_hi, A);
+        else run_tiles<kTRI6, 2>(tile, J, P, Y0, sign, T, f, s_lo, s_hi, A);
     } else {
-        if (P.oi == 0) run_tiles<kSQ4, 0>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
-        else run_tiles<kSQ4, 1>(tile, J, P, Y0, sign, thr, f, s_lo, s_hi, A);
+        if (P.oi == 0) run_tiles<kSQ4, 0>(tile, J, P, Y0, sign, T, f, s_lo, s_hi, A);
+        else run_tiles<kSQ4, 1>(tile, J, P, Y0, sign, T, f, s_lo, s_hi, A);
     }
 
     const long long att = blockIdx.x == 0 && tid == 0 ? P.att : 0;  // the whole phase's, counted once
