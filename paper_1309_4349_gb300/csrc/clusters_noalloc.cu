@@ -32,7 +32,7 @@ constexpr long long kMaxSites = KLMC_NOALLOC_MAX_SITES;
 
 constexpr unsigned long long align256(unsigned long long v) { return (v + 255ull) & ~255ull; }
 
-// Same carve as cluster_scratch_carve for N = n_species_max = kMaxSites.
+// At least cluster_scratch_bytes(N, N) for every N up to kMaxSites.
 constexpr unsigned long long kScratchBytes =
     2 * align256(4ull * kMaxSites) + align256(4ull * (kMaxSites + 1)) +
     align256(4ull * ((kMaxSites + 1 + 31) / 32));

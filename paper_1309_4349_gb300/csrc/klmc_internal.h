@@ -154,12 +154,17 @@ cudaError_t launch_unpack(const void *lat, int packing, int Lx, int Ly, int pitc
 cudaError_t launch_count_A(const void *lat, int packing, int Lx, int Ly, int pitch, long long *out,
                            cudaStream_t stream);
 
-// Cluster histogram scratch for n sites and up to n_species sites of one species.
+// Cluster histogram scratch for lattices of up to n sites (of any shape) and up to
+// n_species sites of one species.  hist .. zero_end is zero between calls.
 struct ClusterScratch {
-    int32_t *parent;      // [N]
-    int32_t *csize;       // [N]
-    int32_t *hist;        // [n_species + 1], zero between calls
-    uint32_t *bitmap;     // [(n_species + 1 + 31) / 32], zero between calls
+    int32_t *hist;              // [n_species + 1] clusters of a size
+    uint32_t *l0, *l1, *l2;     // occupied sizes, 1 bit each; occupied words of l0, of l1
+    uint32_t *done;             // CTAs of the counting launch that have finished
+    void *zero_end;
+    int32_t *parent, *csize;    // tree and sizes of the components at tile borders
+    int32_t *labels;            // their nodes at the tiles' border sites
+    int32_t *nodes;             // nodes of each tile
+    void *end;
     long long n_species_max;
 };
 size_t cluster_scratch_bytes(long long N, long long n_species_max);
