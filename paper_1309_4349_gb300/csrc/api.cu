@@ -48,13 +48,15 @@ bool device_ok(std::string *why)
         *why = "cudaGetDevice failed";
         return false;
     }
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) {
-        *why = "cudaGetDeviceProperties failed";
+    // (attributes, not cudaGetDeviceProperties: this runs in every create)
+    int major = 0, minor = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess) {
+        *why = "cudaDeviceGetAttribute failed";
         return false;
     }
-    if (prop.major * 10 + prop.minor != 103) {
-        *why = "library built for sm_103a; device is sm_" + std::to_string(prop.major * 10 + prop.minor);
+    if (major * 10 + minor != 103) {
+        *why = "library built for sm_103a; device is sm_" + std::to_string(major * 10 + minor);
         return false;
     }
     return true;
@@ -341,11 +343,11 @@ klmc_status create_one(klmc_ctx **out, const klmc_params *p, klmc_batch *owner, 
     // writer writes sites only, or whole rows with zero padding.
     if (e == cudaSuccess) e = cudaMemsetAsync(c->lat, 0, c->lat_bytes, c->stream);
     if (e == cudaSuccess)
-        e = launch_init_lattice(c->lat, J.packing, p->Lx, p->Ly, c->pitch, J.key0, J.key1, c->nA,
+        e = launch_init_lattice(c->lat, c->lat_bytes, J.packing, p->Lx, p->Ly, c->pitch, J.key0, J.key1, c->nA,
                                 c->init_scratch, c->stream);
     if (e == cudaSuccess)
-        e = launch_recount(c->lat, J.packing, p->Lx, p->Ly, c->pitch, p->geometry,
-                           c->state + kNUnlike, c->stream, c->helical);
+        e = launch_tally(c->lat, J.packing, p->Lx, p->Ly, c->pitch, p->geometry, c->helical, c->state + kNUnlike,
+                         nullptr, c->stream);  // (the state was zeroed above)
     if (e == cudaSuccess && sync) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         free_all(c);
@@ -1060,10 +1062,8 @@ klmc_status klmc_set_lattice(klmc_ctx *c, const uint8_t *host_in, int64_t n, int
     KLMC_CUDA(cudaMemcpyAsync(c->dbytes, host_in, (size_t)n, cudaMemcpyHostToDevice, c->stream));
     KLMC_CUDA(launch_pack(c->dbytes, c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->stream));
     KLMC_CUDA(cudaMemsetAsync(c->state, 0, kStateSlots * sizeof(long long), c->stream));
-    KLMC_CUDA(launch_recount(c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->p.geometry,
-                             c->state + kNUnlike, c->stream, c->helical));
-    KLMC_CUDA(launch_count_A(c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->state + kScratch0,
-                             c->stream));
+    KLMC_CUDA(launch_tally(c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->p.geometry, c->helical,
+                           c->state + kNUnlike, c->state + kScratch0, c->stream));
     long long nA = 0;
     KLMC_CUDA(cudaMemcpyAsync(&nA, c->state + kScratch0, sizeof(nA), cudaMemcpyDeviceToHost, c->stream));
     KLMC_CUDA(cudaStreamSynchronize(c->stream));
@@ -1081,10 +1081,8 @@ klmc_status klmc_set_lattice_device(klmc_ctx *c, const uint8_t *dev_in, int64_t 
     if (sweep_index < 0) return fail(KLMC_EINVAL, "sweep_index must be >= 0");
     KLMC_CUDA(launch_pack(dev_in, c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->stream));
     KLMC_CUDA(cudaMemsetAsync(c->state, 0, kStateSlots * sizeof(long long), c->stream));
-    KLMC_CUDA(launch_recount(c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->p.geometry,
-                             c->state + kNUnlike, c->stream, c->helical));
-    KLMC_CUDA(launch_count_A(c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->state + kNA,
-                             c->stream));
+    KLMC_CUDA(launch_tally(c->lat, c->job.packing, c->p.Lx, c->p.Ly, c->pitch, c->p.geometry, c->helical,
+                           c->state + kNUnlike, c->state + kNA, c->stream));
     c->nA_on_device = true;
     c->sweep = sweep_index;
     return KLMC_OK;

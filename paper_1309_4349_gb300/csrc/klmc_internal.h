@@ -135,8 +135,8 @@ size_t helical_resident_smem_bytes(int Lx, int Ly, int cluster);
 cudaError_t launch_helical_resident(const SweepJob &job, const SweepCall &call, int cluster, cudaStream_t stream);
 cudaError_t launch_mpkk_phases(const SweepJob &job, int k0, int n_sweeps, int sm_count, cudaStream_t stream);
 
-// Initial placement: the nA sites with the smallest (64-bit Philox key, index).
-cudaError_t launch_init_lattice(void *lat, int packing, int Lx, int Ly, int pitch, uint32_t key0,
+// Initial placement into a zeroed store: the nA sites with the smallest (64-bit Philox key, index).
+cudaError_t launch_init_lattice(void *lat, size_t lat_bytes, int packing, int Lx, int Ly, int pitch, uint32_t key0,
                                 uint32_t key1, long long nA, void *scratch, cudaStream_t stream);
 size_t init_scratch_bytes();
 
@@ -150,9 +150,9 @@ cudaError_t launch_pack(const uint8_t *bytes, void *lat, int packing, int Lx, in
                         cudaStream_t stream);
 cudaError_t launch_unpack(const void *lat, int packing, int Lx, int Ly, int pitch, uint8_t *bytes,
                           cudaStream_t stream);
-// Count of A sites into *out (overwritten).
-cudaError_t launch_count_A(const void *lat, int packing, int Lx, int Ly, int pitch, long long *out,
-                           cudaStream_t stream);
+// Adds the lattice's unlike bonds to *unlike and its A sites to *sites_A (either may be null).
+cudaError_t launch_tally(const void *lat, int packing, int Lx, int Ly, int pitch, int geometry, int helical,
+                         long long *unlike, long long *sites_A, cudaStream_t stream);
 
 // Cluster histogram scratch for lattices of up to n sites (of any shape) and up to
 // n_species sites of one species.  hist .. zero_end is zero between calls.
