@@ -129,7 +129,7 @@ klmc_status klmc_create_ex(klmc_ctx **out, const klmc_params *p);
  * (cluster = 0) a lattice of at least 786432 sites (where the tiled path measured
  * faster) or too large for one thread-block cluster's shared memory runs on the
  * tiled path (replicas of a batch and jobs of a server stay resident): bands of
- * rows, one CTA each, four phases per launch,
+ * rows, one CTA each, four or eight phases per launch,
  * rows of a bit store on 16-byte boundaries moved by bulk copies.  With an explicit
  * cluster size, EINVAL when the lattice does not fit it (each CTA's band of padded
  * bit rows plus its halo rows must fit its shared memory). */

@@ -100,7 +100,7 @@ TiledPlan tiled_band_plan(int Lx, int Ly, int sm_count);
 cudaError_t configure_tiled();
 cudaError_t configure_band();
 cudaError_t launch_band_phases(const SweepJob &job, const TiledPlan &plan, const void *src, void *dst,
-                               int k, int f0, cudaStream_t stream);
+                               int k, int f0, bool first, cudaStream_t stream);
 // Sweeps k0 .. k0 + n_sweeps - 1 of the plan.  With K >= 2 the launches alternate
 // between job.lat and alt (lat_bytes each) and end in job.lat (a copy back after
 // an odd number of launches).

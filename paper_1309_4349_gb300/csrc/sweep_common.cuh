@@ -254,23 +254,33 @@ __device__ __forceinline__ WordEnds word_ends(int j, int W, int nlast, int hrow)
     return E;
 }
 
+// How a word's windows are taken: kPlain, the words beside it are its neighbours (one funnel
+// shift per window); kEnds, it may be at an end of its row; kFix, and rows may have a last
+// word of one site.
+enum Windows { kPlain, kEnds, kFix };
+
 // The sites at distance -1, +1 and +2 of the word at p (32 at a time).
+template <Windows WN>
 __device__ __forceinline__ uint32_t window_m1(const uint32_t *p, const WordEnds &E)
 {
+    if (WN == kPlain) return __funnelshift_r(p[-1], p[0], 31);
     return p[0] + p[0] + (p[E.l] >> E.top);  // bits above the left word's last site are zero
 }
+template <Windows WN>
 __device__ __forceinline__ uint32_t window_p1(const uint32_t *p, const WordEnds &E)
 {
+    if (WN == kPlain) return __funnelshift_r(p[0], p[1], 1);
     return (p[0] >> 1) + p[E.r] * (1u << E.end);
 }
-template <bool FIX>
+template <Windows WN>
 __device__ __forceinline__ uint32_t window_p2(const uint32_t *p, const WordEnds &E)
 {
+    if (WN == kPlain) return __funnelshift_r(p[0], p[1], 2);
     const uint32_t r = p[E.r];
     uint32_t v = (p[0] >> 2) + r * ((1u << E.end) >> 1);
-    // the sum's bits past the row's end carry nothing into it; with a last word of one
-    // site, that word's site and the last one before it look two words on
-    if (FIX && E.fix) v = E.end == 0 ? r >> 1 : (v & 0x7FFFFFFFu) | (p[E.fix2] << 31);
+    // (the sum's bits past the row's end carry nothing into it; with a last word of one
+    // site, that word's site and the last one before it look two words on)
+    if (WN == kFix && E.fix) v = E.end == 0 ? r >> 1 : (v & 0x7FFFFFFFu) | (p[E.fix2] << 31);
     return v;
 }
 
@@ -279,48 +289,51 @@ __device__ __forceinline__ uint32_t window_p2(const uint32_t *p, const WordEnds 
 // the bit planes of S.  A pair that moves is unlike, so a neighbour of both sites is
 // like exactly one of them and adds a constant: only the six neighbours of one site
 // alone are compared (10 comparisons and adders of 10 inputs before, 6 now).
-// FIX: rows may have a last word of one site.
-template <int G, int OI, bool FIX>
+template <int G, int OI, Windows WN>
 __device__ __forceinline__ void evaluate(const uint32_t *p, int RW, const WordEnds &E, uint32_t &ta, uint32_t &tb,
                                          Planes &S)
 {
     const uint32_t *pm = p - RW, *pp = p + RW;
     ta = p[0];
-    const uint32_t Am = window_m1(p, E);
+    const uint32_t Am = window_m1<WN>(p, E);
     if (G == kTRI6 && OI == 0) {
         // a: (-1,0) (0,-1) (-1,1); b = (1,0): (2,0) (1,1) (2,-1); common (0,1) (1,-1)
-        tb = window_p1(p, E);
-        S = count_unlike(ta, Am, pm[0], window_m1(pp, E), window_p2<FIX>(p, E), window_p1(pp, E), window_p2<FIX>(pm, E));
+        tb = window_p1<WN>(p, E);
+        S = count_unlike(ta, Am, pm[0], window_m1<WN>(pp, E), window_p2<WN>(p, E), window_p1<WN>(pp, E), window_p2<WN>(pm, E));
     } else if (G == kTRI6 && OI == 1) {
         // a: (-1,0) (0,-1) (1,-1); b = (0,1): (1,1) (0,2) (-1,2); common (1,0) (-1,1)
         const uint32_t *pq = pp + RW;
         tb = pp[0];
-        S = count_unlike(ta, Am, pm[0], window_p1(pm, E), window_p1(pp, E), pq[0], window_m1(pq, E));
+        S = count_unlike(ta, Am, pm[0], window_p1<WN>(pm, E), window_p1<WN>(pp, E), pq[0], window_m1<WN>(pq, E));
     } else if (G == kTRI6 && OI == 2) {
         // a: (-1,0) (0,1) (-1,1); b = (1,-1): (2,-1) (1,-2) (2,-2); common (1,0) (0,-1)
         const uint32_t *pn = pm - RW;
-        tb = window_p1(pm, E);
-        S = count_unlike(ta, Am, pp[0], window_m1(pp, E), window_p2<FIX>(pm, E), window_p1(pn, E), window_p2<FIX>(pn, E));
+        tb = window_p1<WN>(pm, E);
+        S = count_unlike(ta, Am, pp[0], window_m1<WN>(pp, E), window_p2<WN>(pm, E), window_p1<WN>(pn, E), window_p2<WN>(pn, E));
     } else if (G == kSQ4 && OI == 0) {
         // a: (-1,0) (0,1) (0,-1); b = (1,0): (2,0) (1,1) (1,-1)
-        tb = window_p1(p, E);
-        S = count_unlike(ta, Am, pp[0], pm[0], window_p2<FIX>(p, E), window_p1(pp, E), window_p1(pm, E));
+        tb = window_p1<WN>(p, E);
+        S = count_unlike(ta, Am, pp[0], pm[0], window_p2<WN>(p, E), window_p1<WN>(pp, E), window_p1<WN>(pm, E));
     } else {
         // SQ4; a: (1,0) (-1,0) (0,-1); b = (0,1): (1,1) (-1,1) (0,2)
         tb = pp[0];
-        S = count_unlike(ta, window_p1(p, E), Am, pm[0], window_p1(pp, E), window_m1(pp, E), pp[RW]);
+        S = count_unlike(ta, window_p1<WN>(p, E), Am, pm[0], window_p1<WN>(pp, E), window_m1<WN>(pp, E), pp[RW]);
     }
 }
 
 // Partners b = a + o of the accepted anchors acc of a word with ends E: their mask in
 // the word at the same place of b's row, and (returned) the one that falls into the
 // word on its right, as its bit 0.
-template <int OI>
+template <int OI, Windows WN = kEnds>
 __device__ __forceinline__ uint32_t partners(uint32_t acc, const WordEnds &E, uint32_t &b)
 {
     if (OI == 1) {
         b = acc;
         return 0u;
+    }
+    if (WN == kPlain) {
+        b = acc << 1;
+        return acc >> 31;
     }
     b = (acc << 1) & (2u * (1u << E.end) - 1u);
     return (acc >> E.end) & 1u;
@@ -375,8 +388,10 @@ __device__ __forceinline__ void draw_accepts_queue2(uint32_t dmask0, const Plane
 {
     acc0 = 0u;
     acc1 = 0u;
-    dmask0 &= ~never_accepted(S0.s0, S0.s1, T.never);
-    dmask1 &= ~never_accepted(S1.s0, S1.s1, T.never);
+    if (T.never != 0u) {
+        dmask0 &= ~never_accepted(S0.s0, S0.s1, T.never);
+        dmask1 &= ~never_accepted(S1.s0, S1.s1, T.never);
+    }
     if (!__any_sync(0xFFFFFFFFu, (dmask0 | dmask1) != 0u)) return;
     const int lane = (int)(threadIdx.x & 31);
     const int nd0 = __popc(dmask0), nd = nd0 + __popc(dmask1);

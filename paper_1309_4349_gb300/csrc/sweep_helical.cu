@@ -157,7 +157,7 @@ __device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGe
         uint32_t ta, tb;
         Planes S;
         const WordEnds E = word_ends(j, g.W, g.nlast, g.RW);
-        evaluate<kTRI6, OI, true>(lat + lr * g.RW + j, g.RW, E, ta, tb, S);
+        evaluate<kTRI6, OI, kFix>(lat + lr * g.RW + j, g.RW, E, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
         const uint32_t dmask = unl & draw_positions(S, g.sign);
         uint32_t acc = unl & ~dmask;

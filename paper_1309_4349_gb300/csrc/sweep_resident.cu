@@ -94,6 +94,7 @@ struct Geo {
     int base;            // (Y0 - D) mod Ly
     int tabW;            // words of a table's anchor masks (even)
     int nlast;           // sites of a row's last word
+    uint32_t magicInner;  // as magicW for the words of a row without its kEndCount end words (band kernel)
 };
 
 __device__ __forceinline__ int task_row(const Geo &g, int t)
@@ -103,20 +104,20 @@ __device__ __forceinline__ int task_row(const Geo &g, int t)
 
 // Flips, in this CTA's rows, the accepted anchors acc of the word at shared address wa
 // and their partners.  Atomics of 0 cost less than branches around them.
-template <int OI>
+template <int OI, Windows WN = kEnds>
 __device__ __forceinline__ void flip_pairs(uint32_t wa, int RW, const WordEnds &E, uint32_t acc)
 {
     const uint32_t rowbytes = 4u * (uint32_t)RW;
     const uint32_t wb = OI == 0 ? wa : (OI == 1 ? wa + rowbytes : wa - rowbytes);
     uint32_t b;
-    const uint32_t next = partners<OI>(acc, E, b);
+    const uint32_t next = partners<OI, WN>(acc, E, b);
     if (OI == 0) {
         red_xor_local(wa, acc | b);
     } else {
         red_xor_local(wa, acc);
         red_xor_local(wb, b);
     }
-    if (OI != 1) red_xor_local(wb + 4u * (uint32_t)E.r, next);
+    if (OI != 1) red_xor_local(WN == kPlain ? wb + 4u : wb + 4u * (uint32_t)E.r, next);
 }
 
 // Flips m in word j of global row r (unwrapped, in [Y0 - 1, Y1]) in every CTA holding a copy.
@@ -281,7 +282,7 @@ __device__ __forceinline__ Task load_task(const uint32_t *lat, const Geo &g, int
 // of one or two warps per scheduler), so a phase lasts as long as the instruction
 // stream of its busiest warp.  Branches in it cost most: the geometry, the orientation
 // and the rare row shapes are template parameters.
-template <int G, int OI, int NT, bool BLOCKED, bool FIX>
+template <int G, int OI, int NT, bool BLOCKED, Windows WN>
 __device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, const PhaseHdr &h, Task k,
                                           const PhaseR &P, const DrawThr &T, const DrawKey &dk, Acc &A,
                                           bool use_tab, const uint32_t *tab)
@@ -292,7 +293,7 @@ __device__ __forceinline__ void run_phase(const uint32_t *lat, const Geo &g, con
     for (int tl = threadIdx.x; tl < h.nlane;) {
         uint32_t ta, tb;
         Planes S;
-        evaluate<G, OI, FIX>(k.p, g.RW, k.E, ta, tb, S);
+        evaluate<G, OI, WN>(k.p, g.RW, k.E, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & k.am;
         const uint32_t dmask = unl & draw_positions(S, g.sign);
         const uint32_t acc = (unl & ~dmask) | draw_accepts(dmask, S, k.site, dk, T);
@@ -330,16 +331,32 @@ struct TaskPrep {
     bool own;
 };
 
-template <int G, int OI>
+// Which words of the anchor rows a loop of tasks takes: all, those away from the rows' ends
+// (plain windows), or the first and the last two.
+enum RowPart { kAllWords, kInnerWords, kEndWords };
+constexpr int kEndCount = 3;
+
+template <int G, int OI, RowPart RP>
 __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g, const PhaseR &P, bool use_tab,
                                                const TaskTab *tt, int t, bool valid, TaskPrep &T, Acc &A)
 {
+    constexpr Windows WN = RP == kInnerWords ? kPlain : kFix;
     uint32_t am = 0u, ta = 0u, tb = 0u;
     Planes S = {0u, 0u, 0u};
     int ybase = 0, j = 0, lr = 0;
     if (valid) {
-        const int mi = task_row(g, t);
-        j = t - mi * g.W;
+        int mi;
+        if (RP == kInnerWords) {
+            mi = (int)__umulhi((uint32_t)t, g.magicInner);
+            j = t - mi * (g.W - kEndCount) + 1;
+        } else if (RP == kEndWords) {
+            mi = t / kEndCount;
+            j = t - mi * kEndCount;
+            j = j == 0 ? 0 : g.W - kEndCount + j;
+        } else {
+            mi = task_row(g, t);
+            j = t - mi * g.W;
+        }
         if (use_tab) {
             const int2 r = tt->row[mi];
             lr = r.x;
@@ -355,7 +372,7 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
             ybase = y * g.Lx;
             am = anchor_mask(j << 5, P, g.Lx);
         }
-        evaluate<G, OI, true>(lat + lr * g.RW + j, g.RW, word_ends(j, g.W, g.nlast, 0), ta, tb, S);
+        evaluate<G, OI, WN>(lat + lr * g.RW + j, g.RW, word_ends(j, g.W, g.nlast, 0), ta, tb, S);
     }
     const uint32_t unl = (ta ^ tb) & am;
     T.dmask = unl & draw_positions(S, g.sign);
@@ -371,7 +388,7 @@ __device__ __forceinline__ void band_task_prep(const uint32_t *lat, const Geo &g
     }
 }
 
-template <int OI>
+template <int OI, RowPart RP>
 __device__ __forceinline__ void band_task_finish(const Geo &g, const TaskPrep &T, uint32_t acc, Acc &A)
 {
     if (!acc) return;
@@ -380,39 +397,54 @@ __device__ __forceinline__ void band_task_finish(const Geo &g, const TaskPrep &T
         A.acc += na;
         A.dn += half_dn(T.S, acc, na);
     }
-    flip_pairs<OI>(g.lat_addr + 4u * (uint32_t)(T.lr * g.RW + T.j), g.RW, word_ends(T.j, g.W, g.nlast, 0), acc);
+    flip_pairs<OI, RP == kInnerWords ? kPlain : kFix>(g.lat_addr + 4u * (uint32_t)(T.lr * g.RW + T.j), g.RW, word_ends(T.j, g.W, g.nlast, 0), acc);
 }
 
-template <int G, int OI, int THREADS>
+// INNER: wide rows.  Their words away from the ends need no distances around them (7% of
+// a phase of 8192^2); the end words go first, to the last warps, which have the fewest
+// others.
+template <int G, int OI, int THREADS, bool INNER>
 __device__ __forceinline__ void run_phase_pair(const uint32_t *lat, const Geo &g, const PhaseR &P,
                                                const DrawThr &T, int f, uint32_t s_lo, uint32_t s_hi,
                                                Acc &A, uint32_t *q, const TaskTab *tt, const uint32_t (&rk)[2][8])
 {
+    constexpr RowPart RP = INNER ? kInnerWords : kAllWords;
     const int lane = threadIdx.x & 31;
-    const int ntask = P.ntask;
+    const int ntask = INNER ? P.c[3] * (g.W - kEndCount) : P.ntask;
     const bool use_tab = tt != nullptr && table_fits(g, P, *tt);
     const DrawKey dk = draw_key((uint32_t)f, s_lo, s_hi, g.k0, g.k1);
+    if (INNER) {
+        for (int t = THREADS - 32 - (int)(threadIdx.x & ~31) + lane; t < kEndCount * P.c[3]; t += THREADS) {
+            TaskPrep T0;
+            band_task_prep<G, OI, kEndWords>(lat, g, P, use_tab, tt, t, true, T0, A);
+            band_task_finish<OI, kEndWords>(g, T0, T0.acc | draw_accepts(T0.dmask, T0.S, T0.base, dk, T), A);
+        }
+        __syncwarp();
+    }
     for (int t0 = threadIdx.x & ~31; t0 < ntask; t0 += 2 * THREADS) {
         const int ta = t0 + lane, tb = t0 + THREADS + lane;
         TaskPrep T0, T1;
-        band_task_prep<G, OI>(lat, g, P, use_tab, tt, ta, ta < ntask, T0, A);
-        band_task_prep<G, OI>(lat, g, P, use_tab, tt, tb, tb < ntask, T1, A);
+        band_task_prep<G, OI, RP>(lat, g, P, use_tab, tt, ta, ta < ntask, T0, A);
+        band_task_prep<G, OI, RP>(lat, g, P, use_tab, tt, tb, tb < ntask, T1, A);
         uint32_t a0, a1;
         draw_accepts_queue2(T0.dmask, T0.S, T0.base, T1.dmask, T1.S, T1.base, dk, rk, T, q, a0, a1);
-        band_task_finish<OI>(g, T0, T0.acc | a0, A);
-        band_task_finish<OI>(g, T1, T1.acc | a1, A);
+        band_task_finish<OI, RP>(g, T0, T0.acc | a0, A);
+        band_task_finish<OI, RP>(g, T1, T1.acc | a1, A);
     }
 }
 
-template <int G, int THREADS>
+template <int G, int THREADS, bool INNER>
 __device__ __forceinline__ void run_phase_pair_oi(const uint32_t *lat, const Geo &g, const PhaseR &P,
                                                   const DrawThr &T, int f, uint32_t s_lo, uint32_t s_hi,
                                                   Acc &A, uint32_t *q, const TaskTab *tt, const uint32_t (&rk)[2][8])
 {
-    if (P.oi == 0) run_phase_pair<G, 0, THREADS>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
-    else if (G == kTRI6 && P.oi == 2) run_phase_pair<G, 2, THREADS>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
-    else run_phase_pair<G, 1, THREADS>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
+    if (P.oi == 0) run_phase_pair<G, 0, THREADS, INNER>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
+    else if (G == kTRI6 && P.oi == 2) run_phase_pair<G, 2, THREADS, INNER>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
+    else run_phase_pair<G, 1, THREADS, INNER>(lat, g, P, T, f, s_lo, s_hi, A, q, tt, rk);
 }
+
+// Rows of at least this many words have their end words apart.
+constexpr int kInnerRowWords = 96;
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)
@@ -697,7 +729,8 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     Exchange X = {smem_addr(&xbar[0]), 0u, 0u, kExchangePolls, false};
     auto run_tasks = [&](auto geometry, auto is_blocked, auto has_fix) {
         constexpr int G = decltype(geometry)::value;
-        constexpr bool BLOCKED = decltype(is_blocked)::value, FIX = decltype(has_fix)::value;
+        constexpr bool BLOCKED = decltype(is_blocked)::value;
+        constexpr Windows WN = decltype(has_fix)::value ? kFix : kEnds;
         int block = 0;
         for (long long it = 0; it < Cl.n_mcs; ++it) {
             const bool last = it + 1 == Cl.n_mcs;
@@ -719,9 +752,9 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
                     dk.la = h.la;
                     const int oi = h.code & 3;
                     const PhaseR &P = pp[buf][q];
-                    if (oi == 0) run_phase<G, 0, NT, BLOCKED, FIX>(lat, g, h, k, P, T, dk, A, tables, tab);
-                    else if (G == kSQ4 || oi == 1) run_phase<G, 1, NT, BLOCKED, FIX>(lat, g, h, k, P, T, dk, A, tables, tab);
-                    else run_phase<G, 2, NT, BLOCKED, FIX>(lat, g, h, k, P, T, dk, A, tables, tab);
+                    if (oi == 0) run_phase<G, 0, NT, BLOCKED, WN>(lat, g, h, k, P, T, dk, A, tables, tab);
+                    else if (G == kSQ4 || oi == 1) run_phase<G, 1, NT, BLOCKED, WN>(lat, g, h, k, P, T, dk, A, tables, tab);
+                    else run_phase<G, 2, NT, BLOCKED, WN>(lat, g, h, k, P, T, dk, A, tables, tab);
                     if (q < kChunk - 1) {  // the next phase's entry does not wait for this one
                         tab += tab_words;
                         h = hp[q + 1];
@@ -886,6 +919,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     g.nlast = g.Lx - 32 * (g.W - 1);
     g.k0 = J.key0; g.k1 = J.key1;
     g.sign = J.draw_lo > J.draw_hi ? 0 : (J.draw_lo == 0 ? -1 : 1);
+    g.magicInner = g.W > 3 + 1 ? 0xFFFFFFFFu / (uint32_t)(g.W - 3) + 1u : 0u;
     g.tri = J.geometry == kTRI6;
     g.C = (int)gridDim.x;
     g.rank = (int)blockIdx.x;
@@ -909,12 +943,32 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    // Everything below reads what earlier launches on the stream wrote.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const long long s = J.state[kSweepBase] + k;
+    // The block's schedule and task tables need nothing of the launches before it but the
+    // sweep index, which no launch of a series writes (the first launch of a series follows
+    // its writers in full): a CTA whose SM is free prepares them while the previous launch's
+    // last CTAs run.  The tables follow the rows and the draw queues.
+    const long long s = __ldcg(&J.state[kSweepBase]) + k;
     const uint32_t s_lo = (uint32_t)(unsigned long long)s;
     const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
     if (tid < K) phase_table(g, K, s, f0 + tid, &pp[tid]);
+    __syncthreads();
+    const int tab_rows = band_table_rows(H, K);
+    const int tab_w = (g.W + 1) & ~1;  // even, so that the int2 row entries stay aligned
+    uint32_t *const tab_base = smem + band_table_offset(H, K, RWb);
+    if (tables) {
+        for (int q = 0; q < K; ++q) {
+            const PhaseR P = pp[q];
+            uint32_t *const t = tab_base + (size_t)q * (tab_w + 2 * tab_rows);
+            const TaskTab T = {t, (int2 *)(t + tab_w), g.W, tab_rows};
+            build_task_table<true>(P, g, T, tid, THREADS);
+        }
+    }
+    // the warps' draw queues follow the rows (H + 2D rows of the tallest band)
+    uint32_t *const dq = smem + (size_t)(H + 2 * g.D) * RWb + (size_t)(tid >> 5) * kDrawQueue2Words;
+    dq[kDrawQueue2Acc + (tid & 31)] = 0u;  // the queue's accept words start at zero
+    dq[kDrawQueue2Acc + 32 + (tid & 31)] = 0u;
+    // Everything below reads what earlier launches on the stream wrote.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (bulk) {
         // One bulk copy per row (pitch words, 16-byte aligned at both ends) into the
@@ -964,34 +1018,21 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
         }
     }
     __syncthreads();
-    // The block's task tables follow the rows and the draw queues.
-    const int tab_rows = band_table_rows(H, K);
-    const int tab_w = (g.W + 1) & ~1;  // even, so that the int2 row entries stay aligned
-    uint32_t *const tab_base = smem + band_table_offset(H, K, RWb);
-    if (tables) {
-        for (int q = 0; q < K; ++q) {
-            uint32_t *const t = tab_base + (size_t)q * (tab_w + 2 * tab_rows);
-            const TaskTab T = {t, (int2 *)(t + tab_w), g.W, tab_rows};
-            build_task_table<true>(pp[q], g, T, tid, THREADS);
-        }
-        __syncthreads();
-    }
 
     Acc A = {0u, 0u, 0u, 0};
     const DrawThr DT = draw_thresholds(J);
-    // the warps' draw queues follow the rows (H + 2D rows of the tallest band)
-    uint32_t *const dq = smem + (size_t)(H + 2 * g.D) * RWb + (size_t)(tid >> 5) * kDrawQueue2Words;
-    dq[kDrawQueue2Acc + (tid & 31)] = 0u;  // the queue's accept words start at zero
-    dq[kDrawQueue2Acc + 32 + (tid & 31)] = 0u;
     for (int j = 0; j < K; ++j) {
         const PhaseR P = pp[j];
         uint32_t *const t = tab_base + (size_t)j * (tab_w + 2 * tab_rows);
         const TaskTab T = {t, (int2 *)(t + tab_w), g.W, tab_rows};
         const TaskTab *const tt = tables ? &T : nullptr;
-        if (J.geometry == kTRI6)
-            run_phase_pair_oi<kTRI6, THREADS>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
-        else
-            run_phase_pair_oi<kSQ4, THREADS>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+        if (J.geometry == kTRI6) {
+            if (g.W >= kInnerRowWords) run_phase_pair_oi<kTRI6, THREADS, true>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+            else run_phase_pair_oi<kTRI6, THREADS, false>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+        } else {
+            if (g.W >= kInnerRowWords) run_phase_pair_oi<kSQ4, THREADS, true>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+            else run_phase_pair_oi<kSQ4, THREADS, false>(lat, g, P, DT, f0 + j, s_lo, s_hi, A, dq, tt, J.rk);
+        }
         __syncthreads();
     }
 
@@ -1007,7 +1048,6 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
                              ::"l"(to), "r"(from), "r"(row_bytes) : "memory");
             }
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         }
     } else {
         for (int idx = tid; idx < Hc * g.W; idx += THREADS) {
@@ -1036,6 +1076,8 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
             atomicAdd((unsigned long long *)&J.state[slot], (unsigned long long)sum);
         }
     }
+    // The rows' copies have left shared memory (they complete with the launch).
+    if (bulk && tid < 32) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // Three variants: 512 threads (one CTA per SM; single lattices on one CTA), 256
@@ -1162,12 +1204,20 @@ cudaError_t launch_resident_sweep_one(const SweepJob &job, const SweepCall &call
 #endif
 
 
+// Lattices that the automatic choice takes to the tiled path.
+constexpr long long kWideBlockSites = 786432;
+
 TiledPlan tiled_band_plan(int Lx, int Ly, int sm_count)
 {
     TiledPlan p;
     const int RWb = band_row_words((Lx + 31) / 32);
     const long long W = (((Lx + 31) / 32) + 1) & ~1ll;
-    for (int K = KLMC_TILED_BLOCK; K >= 2; K >>= 1) {
+    // Blocks of 8 phases halve the launches, of which each takes 5 us beside its phases; their
+    // wider halos cost nothing while a phase's words, with the halo's, are one per thread
+    // (1447 x 1021 square: 3.3 -> 3.0 us per phase; 8192^2 would lose 5%).
+    const long long Hs = (Ly + sm_count - 1) / sm_count;
+    const bool wide = (long long)Lx * Ly >= kWideBlockSites && (Hs + 2 * 15 + 1) / 2 * ((Lx + 31) / 32) <= kBandThreads;
+    for (int K = wide ? 8 : KLMC_TILED_BLOCK; K >= 2; K >>= 1) {
         const int D = 2 * K + 1;
         long long H = (Ly + sm_count - 1) / sm_count;  // one CTA per SM
         // rows and draw queues must fit: shrink the bands (more bands than SMs)
@@ -1205,10 +1255,11 @@ cudaError_t configure_band()
 }
 
 cudaError_t launch_band_phases(const SweepJob &job, const TiledPlan &plan, const void *src, void *dst,
-                               int k, int f0, cudaStream_t stream)
+                               int k, int f0, bool first, cudaStream_t stream)
 {
     // Programmatic dependent launch: the CTAs of this launch may be scheduled while
-    // the previous one drains, and wait for it in the kernel before reading.
+    // the previous one drains, and wait for it in the kernel before reading.  The first of a
+    // series waits for whatever is before it, as any launch.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((job.Ly + plan.H - 1) / plan.H), 1, 1);
     cfg.blockDim = dim3(kBandThreads, 1, 1);
@@ -1218,7 +1269,7 @@ cudaError_t launch_band_phases(const SweepJob &job, const TiledPlan &plan, const
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = first ? 0 : 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, band_phases_kernel<kBandThreads>, job, src, dst, plan.H, plan.K,
                                        plan.tables, k, f0);
     if (e != cudaSuccess) return e;

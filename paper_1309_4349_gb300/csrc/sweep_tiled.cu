@@ -64,7 +64,7 @@ __device__ __forceinline__ void run_tiles(const uint32_t *tile, const SweepJob &
         uint32_t ta, tb;
         Planes S;
         const WordEnds E = word_ends(j, J.W, J.Lx - 32 * (J.W - 1), 0);
-        evaluate<G, OI, true>(tile + (size_t)(y - Y0 + 2) * J.RW + j, J.RW, E, ta, tb, S);
+        evaluate<G, OI, kFix>(tile + (size_t)(y - Y0 + 2) * J.RW + j, J.RW, E, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
         const uint32_t dmask = unl & draw_positions(S, sign);
         uint32_t acc = unl & ~dmask;
@@ -198,7 +198,7 @@ cudaError_t launch_tiled_phases(const SweepJob &job, const TiledPlan &plan, void
     int launches = 0;
     for (int k = 0; k < n_sweeps; ++k) {
         for (int f0 = 0; f0 < 8; f0 += plan.K) {
-            cudaError_t e = launch_band_phases(job, plan, src, dst, k0 + k, f0, stream);
+            const cudaError_t e = launch_band_phases(job, plan, src, dst, k0 + k, f0, k == 0 && f0 == 0, stream);
             if (e != cudaSuccess) return e;
             void *t = (void *)src;
             src = dst;
