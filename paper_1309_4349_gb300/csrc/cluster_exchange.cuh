@@ -1,0 +1,116 @@
+// cluster_exchange.cuh -- the halo exchange of lattices resident in a thread-block
+// cluster's shared memory, between the CTAs of neighbouring bands.  Included inside
+// namespace klmc by the resident sweeps.
+#pragma once
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p)
+{
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+// Distance from a shared address of this CTA to the same one of CTA `rank`.
+__device__ __forceinline__ uint32_t mapa_distance(uint32_t addr, int rank)
+{
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    return remote - addr;
+}
+
+// Polls of a wait before it gives up; once one has, the launch's other waits poll once.
+constexpr int kExchangePolls = 1 << 20;
+
+// Waits for phase `parity` of the mbarrier at shared address bar, which the stores of
+// another CTA of the cluster complete.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int limit)
+{
+    for (int i = 0; i < limit; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// What a CTA's block exchanges need: its two mbarriers (side 0: from the CTA above,
+// side 1: from the one below) and the distances from its own shared memory to theirs.
+struct Exchange {
+    uint32_t bar, to_prev, to_next;
+    int polls;
+    bool fault;
+};
+
+// End of a block: the D lowest and D highest band rows go to the mailboxes of parity
+// block & 1 in the neighbouring CTAs, by asynchronous stores that count their bytes on
+// the receiver's mbarriers; this CTA's own mailboxes then fill its halo rows.  A CTA
+// waits for its two neighbours only.  Two parities are enough: a neighbour's block
+// n + 2 follows its receipt of this CTA's n + 1, sent after n was read; and the two
+// sides count apart, because one neighbour may be a block ahead of the other.
+// (With a cluster barrier instead, whose release waits for the stores to be
+// acknowledged, an exchange took about 0.8 us of a 400^2 lattice on 16 CTAs.)
+template <int NT>
+__device__ __forceinline__ void exchange_halos(uint32_t *lat, uint32_t lat_addr, int RW, int H, int D, int hmax, int block,
+                                               Exchange &X)
+{
+    const int rw = D * RW;
+    const uint32_t p = (uint32_t)block & 1u;
+    uint32_t *const mbox = lat + (hmax + 2 * D) * RW + 2 * p * rw;
+    const uint32_t mbox_addr = lat_addr + 4u * (uint32_t)((hmax + 2 * D) * RW + 2 * p * rw);
+    if (threadIdx.x < 2) {
+        unsigned long long st;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;"
+                     : "=l"(st) : "r"(X.bar + 8u * threadIdx.x), "r"(4u * (uint32_t)rw) : "memory");
+    }
+    for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
+        const bool low = idx >= rw;  // the lowest rows go up (side 1 there), the highest down (side 0)
+        const uint32_t v = lat[low ? D * RW + idx - rw : H * RW + idx];
+        const uint32_t to = low ? X.to_prev : X.to_next;
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                     ::"r"(mbox_addr + 4u * (uint32_t)idx + to), "r"(v), "r"(X.bar + (low ? 8u : 0u) + to) : "memory");
+    }
+    for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
+        const bool low = idx >= rw;
+        if (!mbar_wait_cluster(X.bar + (low ? 8u : 0u), p, X.polls)) {
+            X.polls = 1;
+            X.fault = true;
+        }
+        lat[low ? (D + H) * RW + idx - rw : idx] = mbox[idx];
+    }
+}
+
+// Readies the two mbarriers (before the cluster barrier that precedes the first exchange).
+__device__ __forceinline__ void exchange_init(unsigned long long *xbar)
+{
+    if (threadIdx.x < 2) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(xbar + threadIdx.x)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+}
+
+__device__ __forceinline__ Exchange exchange_for(const unsigned long long *xbar, uint32_t lat_addr, int C, int rank)
+{
+    return {smem_addr(xbar), mapa_distance(lat_addr, rank == 0 ? C - 1 : rank - 1),
+            mapa_distance(lat_addr, rank + 1 == C ? 0 : rank + 1), kExchangePolls, false};
+}
+
+// By every thread after the last exchange.  A wait that ran out leaves a lattice that is no
+// state of the chain: report it, and give stores in flight a second bounded wait.  No CTA
+// leaves while a peer may still write into it.
+__device__ __forceinline__ void exchange_end(const Exchange &X, long long *state)
+{
+    if (__syncthreads_or(X.fault)) {
+        if (threadIdx.x == 0) atomicExch((unsigned long long *)&state[kFault], 1ull);
+        for (int side = 0; side < 2; ++side)
+            for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * side, par, kExchangePolls);
+    }
+    cluster_barrier();
+}

@@ -4,12 +4,10 @@
 // of a thread-block cluster for the whole launch and evaluated 32 sites per thread.
 //
 // Helical boundary: site i's neighbours are (i + d) mod N for the six axial steps
-// d = dx + dy*Lx.  Read row by row, padded position p of row y holds site
-// (y*Lx + p) mod N: position -1 is the last site of row y-1 and positions Lx,
-// Lx+1 are the first two sites of row y+1.  With these pads in place the
-// bit-sliced evaluation of the periodic kernels applies unchanged, and a flip of
-// site 0, 1 or Lx-1 of a row also flips its copy in the pad of the row above or
-// below.
+// d = dx + dy*Lx.  Read row by row, position p of row y is site (y*Lx + p) mod N:
+// position -1 is the last site of row y-1 and positions Lx, Lx+1 are the first two
+// sites of row y+1.  So the bit-sliced evaluation of the periodic kernels applies
+// with the windows of a row's end words reaching into the rows beside it (WordEnds).
 //
 // Iteration f of sweep s draws the coverage k and one direction d from Philox at
 // {0xFFFFFFFF, f, s_lo, s_hi}; every centre c (c mod 7 = k) attempts the
@@ -24,11 +22,13 @@
 // rows [Y_r, Y_r+1) and holds D = 2K + 1 halo rows per side; it advances K
 // iterations alone, evaluating in the j-th of them the anchors within
 // 2 (K - 1 - j) + 1 rows of its band (a pair's evaluation and its flips reach two
-// rows, and the pads only hold copies of sites in the adjacent rows), and only
-// anchors of its own band are counted.  Then each CTA stores its D lowest and D
-// highest band rows into its neighbours' mailboxes, a cluster barrier follows,
-// the mailboxes fill the halo rows, and every row's pads are recomputed from the
-// rows beside it.  Iterations run across sweep boundaries (seven per sweep).
+// rows, the windows around row ends included), and only anchors of its own band are
+// counted.  Then the halo exchange of cluster_exchange.cuh.  Iterations run across
+// sweep boundaries (seven per sweep).  A thread's first word is the same in every
+// iteration, so its place and ends are found once; the next iteration's schedule entry
+// and draw key are prepared by one lane.  Bound: the instructions of an iteration's
+// busiest warp (402 x 399 on 16 CTAs: 1.26 us per iteration; 1.88 with copies of the row
+// ends and a cluster barrier per exchange).
 #include <string.h>
 
 #include "klmc_internal.h"
@@ -38,11 +38,10 @@ namespace klmc {
 namespace {
 
 #include "sweep_common.cuh"
+#include "cluster_exchange.cuh"
 
 constexpr int kHelicalThreads = 512;
 constexpr int kHelicalMaxSmem = 227 * 1024 - 6144;
-
-__device__ __forceinline__ uint32_t hsmem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void hred_xor(uint32_t addr, uint32_t v)
 {
@@ -61,12 +60,6 @@ __device__ __forceinline__ uint32_t hcluster_ctarank()
     uint32_t v;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(v));
     return v;
-}
-
-__device__ __forceinline__ void hcluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
 template <typename T>
@@ -97,8 +90,21 @@ __host__ __device__ __forceinline__ int helical_block(int Lx, int Ly, int C)
 struct HGeo {
     int Lx, Ly, W, RW, D, H, Y0, C, rank, sign, NL, nlast;
     long long N;
-    unsigned long long magicW;
     uint32_t k0, k1, lat_addr;
+};
+
+// An iteration's schedule entry, prepared one iteration ahead by one lane.
+struct __align__(16) HSched {
+    int oi, kr;       // orientation, anchors' residue mod 7
+    int delta;        // from an anchor to its centre's site
+    uint32_t hk, la;  // the iteration's part of the draw key
+};
+
+// A thread's word of an iteration, relative to the iteration's first row; the same in every
+// iteration.
+struct HWord {
+    int row, j;
+    WordEnds E;
 };
 
 struct HAcc {
@@ -131,68 +137,81 @@ __device__ __forceinline__ uint32_t helical_draws(uint32_t dmask, const Planes &
     return acc & ~never_accepted(S.s0, S.s1, T.never);
 }
 
-// One iteration: anchors of residue kr mod 7 in local rows [lr0, lr0 + nrows),
-// orientation OI, draw counters shifted by delta (the centre of a backward pair).
-template <int OI>
-__device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGeo &g, int kr, int delta,
-                                                  int lr0, int nrows, const DrawKey &dk,
-                                                  const DrawThr &T, HAcc &A)
+__device__ __forceinline__ HWord helical_word(const HGeo &g, int t)
+{
+    HWord w;
+    w.row = t / g.W;
+    w.j = t - w.row * g.W;
+    w.E = word_ends(w.j, g.W, g.nlast, g.RW);
+    return w;
+}
+
+// One iteration: anchors of the entry's residue in local rows [lr0, lr0 + nrows),
+// orientation OI, draw counters shifted to the centres.  w: the thread's first word.
+template <int OI, Windows WN>
+__device__ __forceinline__ void helical_iteration(const uint32_t *lat, const HGeo &g, const HSched &c, int lr0, int nrows,
+                                                  HWord w, const DrawKey &dk, const DrawThr &T, HAcc &A)
 {
     // b = a + o: (1,0) -> same row, +1; (0,1) -> next row; (1,-1) -> previous row, +1
     const uint32_t rowbytes = 4u * (uint32_t)g.RW;
     const int ntask = nrows * g.W;
-    for (int t = (int)threadIdx.x; t < ntask; t += kHelicalThreads) {
-        const int mi = (int)(((unsigned long long)t * g.magicW) >> 32);
-        const int j = t - mi * g.W;
-        const int lr = lr0 + mi;
+    for (int t = (int)threadIdx.x; t < ntask;) {
+        const int lr = lr0 + w.row;
         int y = g.Y0 - g.D + lr;
         y = y < 0 ? y + g.Ly : (y >= g.Ly ? y - g.Ly : y);
-        const int x0 = j << 5;
-        const uint32_t a0 = (uint32_t)y * (uint32_t)g.Lx + (uint32_t)x0;  // site of position 0 (< N < 2^31)
+        const uint32_t a0 = (uint32_t)y * (uint32_t)g.Lx + 32u * (uint32_t)w.j;  // site of position 0 (< N < 2^31)
         // anchors: positions p with (a0 + p) = kr mod 7, below Lx
-        int o = kr - (int)(a0 % 7u);
+        int o = c.kr - (int)(a0 % 7u);
         o += o < 0 ? 7 : 0;
-        uint32_t am = 0x10204081u << o;  // bits o, o+7, o+14, o+21, o+28
-        if (g.Lx - x0 < 32) am &= (1u << (g.Lx - x0)) - 1u;
+        // bits o, o+7, o+14, o+21, o+28; word W-1 ends at bit E.end
+        const uint32_t am = (0x10204081u << o) & (2u * (1u << w.E.end) - 1u);
         uint32_t ta, tb;
         Planes S;
-        const WordEnds E = word_ends(j, g.W, g.nlast, g.RW);
-        evaluate<kTRI6, OI, kFix>(lat + lr * g.RW + j, g.RW, E, ta, tb, S);
+        const uint32_t *const p = lat + lr * g.RW + w.j;
+        evaluate<kTRI6, OI, WN>(p, g.RW, w.E, ta, tb, S);
         const uint32_t unl = (ta ^ tb) & am;
         const uint32_t dmask = unl & draw_positions(S, g.sign);
-        uint32_t acc = unl & ~dmask;
-        acc |= helical_draws(dmask, S, (int)a0 + delta, (int)g.N, dk, T);
-        const bool own = (unsigned)(lr - g.D) < (unsigned)g.H;
-        if (own) {
-            A.unl += __popc(unl);
-            A.drw += __popc(dmask);
-        }
-        if (acc == 0u) continue;
-        if (own) {
-            const int na = __popc(acc);
-            A.acc += na;
-            A.dn += 2 * half_dn(S, acc, na);
-        }
-        const uint32_t wa = g.lat_addr + 4u * (uint32_t)(lr * g.RW + j);
+        const uint32_t acc = (unl & ~dmask) | helical_draws(dmask, S, (int)a0 + c.delta, (int)g.N, dk, T);
+        const uint32_t own = (unsigned)(lr - g.D) < (unsigned)g.H ? ~0u : 0u;
+        const uint32_t oacc = acc & own;
+        const int na = __popc(oacc);
+        A.unl += __popc(unl & own);
+        A.drw += __popc(dmask & own);
+        A.acc += na;
+        A.dn += half_dn(S, oacc, na);
+        const uint32_t wa = smem_addr(p);
         const uint32_t wb = OI == 0 ? wa : (OI == 1 ? wa + rowbytes : wa - rowbytes);
         uint32_t b;
-        const uint32_t next = partners<OI>(acc, E, b);
+        const uint32_t next = partners<OI>(acc, w.E, b);
         if (OI == 0) {
             hred_xor(wa, acc | b);
         } else {
             hred_xor(wa, acc);
             hred_xor(wb, b);
         }
-        if (OI != 1) hred_xor(wb + 4u * (uint32_t)E.r, next);
+        if (OI != 1) hred_xor(wb + 4u * (uint32_t)w.E.r, next);
+        t += kHelicalThreads;
+        if (t < ntask) w = helical_word(g, t);
     }
 }
 
 // Iteration f of sweep s: the colour kc in [0, 7) and the direction draw d in [0, 6)
 // (orientation d / 2, backward pair when d is odd), from the schedule's Philox block.
-__device__ __forceinline__ uint2 helical_sched(const HGeo &g, unsigned long long s, int f)
+__device__ __forceinline__ void helical_sched(const HGeo &g, unsigned long long s, int f, HSched *c)
 {
     const Philox4 w = philox4(0xFFFFFFFFu, (uint32_t)f, (uint32_t)s, (uint32_t)(s >> 32), g.k0, g.k1);
-    return make_uint2(__umulhi(w.v[0], 7u), __umulhi(w.v[1], 6u));
+    const int kc = (int)__umulhi(w.v[0], 7u), d = (int)__umulhi(w.v[1], 6u), oi = d >> 1;
+    const bool back = d & 1;  // a backward pair's centre is its anchor + o
+    // kr = (kc - delta) mod 7, from delta mod 7 in {0, 1, Lx mod 7, 1 - Lx mod 7}
+    const int lx7 = g.Lx % 7;
+    int kr = kc - (back ? (oi == 0 ? 1 : (oi == 1 ? lx7 : (lx7 <= 1 ? 1 - lx7 : 8 - lx7))) : 0);
+    kr += kr < 0 ? 7 : 0;
+    const DrawKey dk = draw_key((uint32_t)f, (uint32_t)s, (uint32_t)(s >> 32), g.k0, g.k1);
+    c->oi = oi;
+    c->kr = kr;
+    c->delta = back ? (oi == 0 ? 1 : (oi == 1 ? g.Lx : 1 - g.Lx)) : 0;
+    c->hk = dk.hk;
+    c->la = dk.la;
 }
 
 __global__ void __launch_bounds__(kHelicalThreads, 1)
@@ -201,11 +220,12 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     constexpr int kWarps = kHelicalThreads / 32;
     extern __shared__ __align__(16) uint32_t lat[];
     __shared__ long long red[5][kWarps];
-    __shared__ uint2 sched[2];  // (colour, direction draw) of the current and the next iteration
+    __shared__ HSched sched[2];  // the current and the next iteration
+    __shared__ __align__(8) unsigned long long xbar[2];
     if (Cl.n_mcs <= 0) return;
 
     HGeo g;
-    g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = J.RW; g.magicW = J.magicW;
+    g.Lx = J.Lx; g.Ly = J.Ly; g.W = J.W; g.RW = J.RW;
     g.k0 = J.key0; g.k1 = J.key1;
     g.N = (long long)J.Lx * J.Ly;
     g.nlast = g.Lx - 32 * (g.W - 1);
@@ -219,7 +239,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     const int K = helical_block(g.Lx, g.Ly, g.C);  // >= 2: the host launches only such lattices
     g.D = 2 * K + 1;
     g.NL = g.H + 2 * g.D;
-    g.lat_addr = hsmem_addr(lat);
+    g.lat_addr = smem_addr(lat);
     const int hmax = (g.Ly + g.C - 1) / g.C;
     const int tid = threadIdx.x;
 
@@ -233,9 +253,9 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     // Iteration f of sweep s draws its colour and direction from one Philox block;
     // the last warp's lane 0 draws them one iteration ahead, off the tasks' path.
     const bool sched_lane = tid == kHelicalThreads - 32;
-    if (sched_lane) sched[0] = helical_sched(g, (unsigned long long)Cl.sweep0, 0);
-    const int lx7 = g.Lx % 7;
-    hcluster_sync();  // every CTA of the cluster runs before any peer writes into it
+    if (sched_lane) helical_sched(g, (unsigned long long)Cl.sweep0, 0, &sched[0]);
+    exchange_init(xbar);
+    cluster_barrier();  // every CTA of the cluster runs before any peer writes into it
 
     const long long n_unlike0 = (tid == 0 && g.rank == 0 && Cl.trace_every > 0) ? J.state[kNUnlike] : 0;
     // Every iteration attempts one exchange per seven sites (7 | N), counted by one thread.
@@ -244,65 +264,40 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     long long t_dn = 0;
     int jb = 0, pb = 0;  // iteration within the block; buffer of the current schedule entry
     int block = 0;
+    Exchange X = exchange_for(xbar, g.lat_addr, g.C, g.rank);
+    const HWord word = helical_word(g, tid);
     for (long long it = 0; it < Cl.n_mcs; ++it) {
-        const long long s = Cl.sweep0 + it;
-        const uint32_t s_lo = (uint32_t)(unsigned long long)s;
-        const uint32_t s_hi = (uint32_t)((unsigned long long)s >> 32);
+        const unsigned long long s = (unsigned long long)(Cl.sweep0 + it);
+        DrawKey dk = draw_key(0u, (uint32_t)s, (uint32_t)(s >> 32), g.k0, g.k1);
         HAcc A = {0u, 0u, 0u, 0};
+#pragma unroll 1
         for (int f = 0; f < 7; ++f) {
-            const uint2 sc = sched[pb];
-            const int kc = (int)sc.x;
-            const int d = (int)sc.y;
-            const int oi = d >> 1;
-            const long long step = oi == 0 ? 1 : (oi == 1 ? g.Lx : 1 - g.Lx);
-            const int delta = (d & 1) ? (int)step : 0;  // backward pair: its centre is anchor + o
-            // kr = (kc - delta) mod 7, from delta mod 7 in {0, 1, Lx mod 7, 1 - Lx mod 7}
-            const int dm7 = (d & 1) ? (oi == 0 ? 1 : (oi == 1 ? lx7 : (lx7 <= 1 ? 1 - lx7 : 8 - lx7))) : 0;
-            int kr = kc - dm7;
-            kr += kr < 0 ? 7 : 0;
+            const HSched c = sched[pb];
+            const bool last = f == 6 && it + 1 == Cl.n_mcs;
+            if (sched_lane && !last) helical_sched(g, f == 6 ? s + 1 : s, f == 6 ? 0 : f + 1, &sched[pb ^ 1]);
+            dk.hk = c.hk;
+            dk.la = c.la;
             const int e = 2 * (K - 1 - jb) + 1;
-            if (sched_lane && !(f == 6 && it + 1 == Cl.n_mcs))
-                sched[pb ^ 1] = f == 6 ? helical_sched(g, (unsigned long long)(s + 1), 0)
-                                       : helical_sched(g, (unsigned long long)s, f + 1);
-            const DrawKey dk = draw_key((uint32_t)f, s_lo, s_hi, g.k0, g.k1);
-            if (oi == 0) helical_iteration<0>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, T, A);
-            else if (oi == 1) helical_iteration<1>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, T, A);
-            else helical_iteration<2>(lat, g, kr, delta, g.D - e, g.H + 2 * e, dk, T, A);
+            if (g.nlast == 1) {  // rows whose last word holds one site take a longer window
+                if (c.oi == 0) helical_iteration<0, kFix>(lat, g, c, g.D - e, g.H + 2 * e, word, dk, T, A);
+                else if (c.oi == 1) helical_iteration<1, kFix>(lat, g, c, g.D - e, g.H + 2 * e, word, dk, T, A);
+                else helical_iteration<2, kFix>(lat, g, c, g.D - e, g.H + 2 * e, word, dk, T, A);
+            } else {
+                if (c.oi == 0) helical_iteration<0, kEnds>(lat, g, c, g.D - e, g.H + 2 * e, word, dk, T, A);
+                else if (c.oi == 1) helical_iteration<1, kEnds>(lat, g, c, g.D - e, g.H + 2 * e, word, dk, T, A);
+                else helical_iteration<2, kEnds>(lat, g, c, g.D - e, g.H + 2 * e, word, dk, T, A);
+            }
             __syncthreads();
             pb ^= 1;
-            const bool last = f == 6 && it + 1 == Cl.n_mcs;
             const bool exch = jb == K - 1;
             jb = exch ? 0 : jb + 1;
             if (exch && !last) {
-                // Exchange: the D lowest and D highest band rows to the neighbours'
-                // mailboxes of parity block & 1, then this CTA's mailboxes into its
-                // halo rows, then every row's pads from the rows beside it.
-                const int rw = g.D * g.RW, p = block & 1;
-                uint32_t *mbox = lat + (size_t)(hmax + 2 * g.D) * g.RW;
-                const uint32_t prev = g.rank == 0 ? g.C - 1 : g.rank - 1;
-                const uint32_t next = g.rank + 1 == g.C ? 0 : g.rank + 1;
-                for (int idx = tid; idx < 2 * rw; idx += kHelicalThreads) {
-                    const int side = idx >= rw ? 1 : 0;
-                    const int k = idx - side * rw;
-                    const uint32_t v = lat[(size_t)(side ? g.D : g.H) * g.RW + k];
-                    const uint32_t local = hsmem_addr(mbox + (size_t)(2 * p + side) * rw + k);
-                    uint32_t remote;
-                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                                 : "=r"(remote) : "r"(local), "r"(side ? prev : next));
-                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
-                }
-                hcluster_sync();
-                for (int idx = tid; idx < 2 * rw; idx += kHelicalThreads) {
-                    const int side = idx >= rw ? 1 : 0;
-                    const int k = idx - side * rw;
-                    lat[(size_t)(side ? g.D + g.H : 0) * g.RW + k] = mbox[(size_t)(2 * p + side) * rw + k];
-                }
+                exchange_halos<kHelicalThreads>(lat, g.lat_addr, g.RW, g.H, g.D, hmax, block++, X);
                 __syncthreads();
-                ++block;
             }
         }
         t_unl += A.unl; t_drw += A.drw; t_acc += A.acc;
-        t_dn += A.dn;
+        t_dn += 2 * A.dn;
         if (Cl.trace_every > 0 && (it + 1) % Cl.trace_every == 0) {
             const long long ws = hwarp_sum(t_dn);
             if ((tid & 31) == 0 && ws != 0)
@@ -312,6 +307,8 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
                           (unsigned long long)n_unlike0);
         }
     }
+
+    exchange_end(X, J.state);
 
     // Write the band back (sites only).
     for (int idx = tid; idx < g.H * g.W; idx += kHelicalThreads) {

@@ -50,11 +50,7 @@ namespace klmc {
 namespace {
 
 #include "sweep_common.cuh"
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
+#include "cluster_exchange.cuh"
 
 // XOR v into the 32-bit word at shared address addr of CTA `rank` of the cluster.
 __device__ __forceinline__ void xor_word(uint32_t addr, uint32_t rank, bool local, uint32_t v)
@@ -147,12 +143,6 @@ __device__ __forceinline__ void flip_global_row(const Geo &g, int r, int j, uint
         if (lr >= g.Ly) lr -= g.Ly;
         for (; lr < Hd + 4; lr += g.Ly) xor_word(word + rowbytes * (uint32_t)lr, (uint32_t)d, d == g.rank, m);
     }
-}
-
-__device__ __forceinline__ void cluster_barrier()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
 // Barrier of the CTA's first NT threads, which run the tasks.
@@ -508,78 +498,6 @@ __device__ __forceinline__ void phase_table(const Geo &g, int K, long long s, in
     phase_ranges(g.tri ? kTRI6 : kSQ4, g.Lx, g.Ly, g.W, g.Y0 - e, g.Y1 + e, g.k0, g.k1, s, f, P);
 }
 
-// Polls of a wait before it gives up; once one has, the launch's other waits poll once.
-constexpr int kExchangePolls = 1 << 20;
-
-// Waits for phase `parity` of the mbarrier at shared address bar, which the stores of
-// another CTA of the cluster complete.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int limit)
-{
-    for (int i = 0; i < limit; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
-// What a CTA's block exchanges need: its two mbarriers (side 0: from the CTA above,
-// side 1: from the one below) and the distances from its own shared memory to theirs.
-struct Exchange {
-    uint32_t bar, to_prev, to_next;
-    int polls;
-    bool fault;
-};
-
-// End of a block: the D lowest and D highest band rows go to the mailboxes of parity
-// block & 1 in the neighbouring CTAs, by asynchronous stores that count their bytes on
-// the receiver's mbarriers; this CTA's own mailboxes then fill its halo rows.  A CTA
-// waits for its two neighbours only.  Two parities are enough: a neighbour's block
-// n + 2 follows its receipt of this CTA's n + 1, sent after n was read; and the two
-// sides count apart, because one neighbour may be a block ahead of the other.
-// (With a cluster barrier instead, whose release waits for the stores to be
-// acknowledged, an exchange took about 0.8 us of a 400^2 lattice on 16 CTAs.)
-template <int NT>
-__device__ __forceinline__ void exchange_halos(uint32_t *lat, const Geo &g, int hmax, int block, Exchange &X)
-{
-    const int H = g.Y1 - g.Y0, D = g.D, rw = D * g.RW;
-    const uint32_t p = (uint32_t)block & 1u;
-    uint32_t *const mbox = lat + (hmax + 2 * D) * g.RW + 2 * p * rw;
-    const uint32_t mbox_addr = g.lat_addr + 4u * (uint32_t)((hmax + 2 * D) * g.RW + 2 * p * rw);
-    if (threadIdx.x < 2) {
-        unsigned long long st;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;"
-                     : "=l"(st) : "r"(X.bar + 8u * threadIdx.x), "r"(4u * (uint32_t)rw) : "memory");
-    }
-    for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
-        const bool low = idx >= rw;  // the lowest rows go up (side 1 there), the highest down (side 0)
-        const uint32_t v = lat[low ? D * g.RW + idx - rw : H * g.RW + idx];
-        const uint32_t to = low ? X.to_prev : X.to_next;
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                     ::"r"(mbox_addr + 4u * (uint32_t)idx + to), "r"(v), "r"(X.bar + (low ? 8u : 0u) + to) : "memory");
-    }
-    for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
-        const bool low = idx >= rw;
-        if (!mbar_wait_cluster(X.bar + (low ? 8u : 0u), p, X.polls)) {
-            X.polls = 1;
-            X.fault = true;
-        }
-        lat[low ? (D + H) * g.RW + idx - rw : idx] = mbox[idx];
-    }
-}
-
-// Distance from a shared address of this CTA to the same one of CTA `rank`.
-__device__ __forceinline__ uint32_t mapa_distance(uint32_t addr, int rank)
-{
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
-    return remote - addr;
-}
-
 // Words of the task tables of one phase, and of the two chunks' (see TaskTab): anchor
 // masks of W words (even, so that the row entries stay aligned) and the rows.
 __host__ __device__ __forceinline__ int phase_table_words(int W, int hmax, int K)
@@ -715,8 +633,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         }
     };
     prepare_chunk(0);
-    if (tid < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&xbar[tid])) : "memory");
-    if (tid < 2) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    exchange_init(xbar);
     // Every CTA of the cluster must be running before any peer writes into it.
     if (C > 1) cluster_barrier();
     else cta_barrier();
@@ -726,7 +643,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     // The preparing warps: the next chunk's tables while the current one runs, then the
     // chunk's last barrier (every phase is a cluster barrier when bands are too thin
     // for blocks).
-    Exchange X = {smem_addr(&xbar[0]), 0u, 0u, kExchangePolls, false};
+    Exchange X = exchange_for(xbar, g.lat_addr, C, rank);
     auto run_tasks = [&](auto geometry, auto is_blocked, auto has_fix) {
         constexpr int G = decltype(geometry)::value;
         constexpr bool BLOCKED = decltype(is_blocked)::value;
@@ -767,7 +684,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
                     // Blocks of K phases end with an exchange, except the launch's last.
                     if (BLOCKED && ((q + 1) & (K - 1)) == 0 && !(last && buf == 1 && q == kChunk - 1)) {
                         task_barrier<NT>();
-                        exchange_halos<NT>(lat, g, hmax, block++, X);
+                        exchange_halos<NT>(lat, g.lat_addr, g.RW, g.Y1 - g.Y0, g.D, hmax, block++, X);
                     }
                     if (q == kChunk - 1) cta_barrier();
                     else task_barrier<NT>();
@@ -798,8 +715,6 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
             }
         }
     } else if (blocked) {
-        X.to_prev = mapa_distance(g.lat_addr, rank == 0 ? C - 1 : rank - 1);
-        X.to_next = mapa_distance(g.lat_addr, rank + 1 == C ? 0 : rank + 1);
         // (rows whose last word holds one site take a longer window: their own copy)
         if (g.nlast == 1) {
             if (g.tri) run_tasks(Const<kTRI6>{}, std::true_type{}, std::true_type{});
@@ -812,17 +727,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         if (g.tri) run_tasks(Const<kTRI6>{}, std::false_type{}, std::true_type{});
         else run_tasks(Const<kSQ4>{}, std::false_type{}, std::true_type{});
     }
-    // A wait that ran out leaves a lattice that is no state of the chain: report it, and
-    // give stores in flight a second bounded wait.  No CTA leaves while a peer may still
-    // write into it.
-    if (blocked) {
-        if (__syncthreads_or(X.fault)) {
-            if (tid == 0) atomicExch((unsigned long long *)&J.state[kFault], 1ull);
-            for (int side = 0; side < 2; ++side)
-                for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * side, par, kExchangePolls);
-        }
-        cluster_barrier();
-    }
+    if (blocked) exchange_end(X, J.state);
 
     // Write the band back (main positions only).
     for (int idx = tid; idx < H * g.W; idx += THREADS) {
