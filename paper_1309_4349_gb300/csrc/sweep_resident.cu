@@ -196,9 +196,6 @@ __device__ __forceinline__ void build_task_table(const PhaseR &P, const Geo &g, 
     }
 }
 
-#ifndef KLMC_SPLIT_LANES
-#define KLMC_SPLIT_LANES(NT) ((NT) > 256 ? 256 : (NT))
-#endif
 // What a phase's tasks need of its schedule entry, prepared with the task table.
 struct __align__(16) PhaseHdr {
     int nlane;        // lanes with tasks: the phase's words, each split over 2^ls lanes
@@ -208,11 +205,13 @@ struct __align__(16) PhaseHdr {
 
 // Lanes per word (log2) of a phase of ntask words on NT threads.  A split word's
 // lanes all evaluate it and each keeps the anchors of its part, which divides the
-// draws (the longest step of a lane) among them.
+// draws (the longest step of a lane) among them.  With 480 task threads the split ends
+// at 192 lanes: more lanes than that cost every scheduler a warp that shares no draws
+// (300^2 on 16 CTAs 1.01 -> 0.99 us per phase, 256^2 0.96 -> 0.95).
 template <int NT>
 __device__ __forceinline__ int word_split(int ntask)
 {
-    constexpr int kLanes = KLMC_SPLIT_LANES(NT);
+    constexpr int kLanes = NT > 256 ? 192 : NT;
     return 4 * ntask <= kLanes ? 2 : (2 * ntask <= kLanes ? 1 : 0);
 }
 
@@ -533,11 +532,12 @@ template <int V>
 using Const = std::integral_constant<int, V>;
 
 // Preparing a phase (a Philox block, the anchor rows' ranges, the tables) takes one
-// warp about 1100 cycles, as long as a phase of a lattice spread over a cluster.  So
-// with more than 128 threads the last kAhead warps do nothing else: they prepare the
+// warp about 600 cycles, half a phase of a lattice spread over a cluster.  So
+// with more than 128 threads the last warp does nothing else: it prepares the
 // next kChunk phases while the others, which synchronise among themselves, run the
-// current ones, and meet them once per chunk.  With 128 threads (several CTAs per SM,
-// every warp busy) each of the four warps prepares one phase of the next chunk before
+// current ones, and meets them once per chunk.  (Two or four such warps were no faster,
+// and took warps from the tasks: 400^2 on 8 CTAs 1.55 us per phase with four, 1.39 with one.)
+// With 128 threads (several CTAs per SM, every warp busy) each of the four warps prepares one phase of the next chunk before
 // its own tasks.
 template <int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB)
@@ -545,7 +545,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
                       const int *__restrict__ job_map, const SweepJob job0, const SweepCall call0)
 {
     constexpr int kWarps = THREADS / 32;
-    constexpr int kAhead = THREADS > 256 ? 4 : (THREADS > 128 ? 2 : 0);
+    constexpr int kAhead = THREADS > 128 ? 1 : 0;
     constexpr int NT = THREADS - 32 * kAhead;  // threads with tasks
     constexpr int kPrep = kAhead > 0 ? kAhead : kWarps;  // warps that prepare
     static_assert(kPrep <= kChunk && kChunk % kPrep == 0, "each preparing warp has kChunk / kPrep phases");
@@ -1068,14 +1068,15 @@ int resident_max_smem_bytes() { return kResidentMaxSmem; }
 int resident_block_phases(int Lx, int Ly, int cluster) { return block_phases(Lx, Ly, cluster); }
 
 // A phase of a lattice spread over a cluster lasts as long as its busiest warp, so the
-// CTA has enough threads for one task each: 192 of 256 or 384 of 512 run tasks (the
-// others prepare).  GB300, us per phase at 256 / 512 threads: 64^2 on 4 CTAs 0.76 /
-// 0.81, 300^2 on 16 1.04 / 1.07, 350^2 1.18 / 1.12, 400^2 1.41 / 1.19.
+// CTA has enough threads for one task each: 224 of 256 or 480 of 512 run tasks (the
+// others prepare).  GB300, us per phase at 256 / 512 threads: 64^2 on 2 CTAs 0.79 /
+// 0.83, 280^2 on 16 0.94 / 0.96, 330^2 on 16 (198 words a phase) 1.04 / 1.04, 262^2 on
+// 8 (216) 1.04 / 1.07, 400^2 on 16 (260) 1.41 / 1.12.
 int resident_default_threads(int Lx, int Ly, int cluster)
 {
     const int C = cluster < 1 ? 1 : cluster, K = block_phases(Lx, Ly, C);
     const int rows = (Ly + C - 1) / C + (K > 1 ? 2 * (2 * K - 1) : 0);
-    return (long long)((rows + 1) / 2) * ((Lx + 31) / 32) > 192 ? 512 : 256;
+    return (long long)((rows + 1) / 2) * ((Lx + 31) / 32) > 224 ? 512 : 256;
 }
 
 int resident_max_cluster(int Ly)
