@@ -1303,7 +1303,9 @@ klmc_status klmc_batch_sweep(klmc_batch *b, const int64_t *n_mcs)
         return KLMC_OK;
     }
     // One launch per launch shape, each on its own stream (the launches overlap on
-    // the GPU), larger lattices first inside a launch.
+    // the GPU), the longest lattices first inside a launch and the shapes with the longest
+    // CTAs first, so that the many small lattices fill the SMs that those leave (GB300, 256
+    // replicas of side 100..1024, 1000 steps: 160 ms with the smallest first, 137 so).
     std::vector<std::pair<int, int>> shapes;
     klmc::host::choose_shapes(active, active_steps, b->sm_count, false, &shapes);
     std::map<std::pair<int, int>, std::vector<int>> groups;
@@ -1311,20 +1313,23 @@ klmc_status klmc_batch_sweep(klmc_batch *b, const int64_t *n_mcs)
         groups[shapes[k]].push_back(index[k]);
         b->last_shape[index[k]] = shapes[k];
     }
+    auto work = [&](int i) { return (double)n_mcs[i] * (double)b->reps[i]->N; };
+    for (auto &g : groups)
+        std::stable_sort(g.second.begin(), g.second.end(), [&](int a, int c) { return work(a) > work(c); });
+    std::vector<std::pair<std::pair<int, int>, std::vector<int>>> order(groups.begin(), groups.end());
+    std::stable_sort(order.begin(), order.end(), [&](const auto &a, const auto &c) {
+        return work(a.second[0]) / a.first.first > work(c.second[0]) / c.first.first;
+    });
     std::vector<int> hmap;
     hmap.reserve(active.size());
-    for (auto &g : groups) {
-        std::stable_sort(g.second.begin(), g.second.end(),
-                         [&](int a, int c) { return b->reps[a]->N > b->reps[c]->N; });
-        hmap.insert(hmap.end(), g.second.begin(), g.second.end());
-    }
+    for (auto &g : order) hmap.insert(hmap.end(), g.second.begin(), g.second.end());
     KLMC_CUDA(cudaMemcpyAsync(b->dcalls, b->hcalls.data(), sizeof(SweepCall) * (size_t)n,
                               cudaMemcpyHostToDevice, b->stream));
     KLMC_CUDA(cudaMemcpyAsync(b->dmap, hmap.data(), sizeof(int) * hmap.size(), cudaMemcpyHostToDevice,
                               b->stream));
     KLMC_CUDA(cudaEventRecord(b->fork, b->stream));  // after the tables' upload
     int offset = 0;
-    for (auto &g : groups) {
+    for (auto &g : order) {
         auto it = b->group_streams.find(g.first);
         if (it == b->group_streams.end()) {
             cudaStream_t gs;
