@@ -77,17 +77,18 @@ ISSUE_LANES_PER_SM = 128
 # each (one resident-sweep launch of 500 MCS of the 400x400 x 5 workload; one
 # 4-phase band launch of the 8192x8192 lattice; one resident helical launch of 500
 # MCS of one 402x399 lattice), valid only for the kernel sources they were taken
-# with (hash of the kernel's file + sweep_common.cuh + philox.cuh).
-TRAFFIC_C2_LAUNCH = 211200
-TRAFFIC_C3_LAUNCH = 8500480
-TRAFFIC_SOURCES = "fabfcfe5f46002be"
-TRAFFIC_C6_LAUNCH = 90624
-TRAFFIC_HELICAL_SOURCES = "4e4cb06710757526"
+# with (hash of the kernel's file + sweep_common.cuh + cluster_exchange.cuh + philox.cuh).
+TRAFFIC_C2_LAUNCH = 230656
+TRAFFIC_C3_LAUNCH = 8494336
+TRAFFIC_SOURCES = "6dd3276ed3228bd1"
+TRAFFIC_C6_LAUNCH = 93184
+TRAFFIC_HELICAL_SOURCES = "56a8f01e6f3bbf26"
 
 # Kernels launched per library call (fixed by the library's structure).
 LAUNCHES_SWEEP = 1
-LAUNCHES_HISTOGRAM = 5
-LAUNCHES_SET_LATTICE_DEVICE = 3
+LAUNCHES_HISTOGRAM = 4
+LAUNCHES_HISTOGRAM_SMALL = 1  # lattices of one CTA's shared memory (64 x 64)
+LAUNCHES_SET_LATTICE_DEVICE = 2
 
 # The other workloads.
 C1 = dict(L=64, n_A=2048, omega=0.6, seed=1, mcs=1000, hist_every=100)
@@ -117,7 +118,7 @@ def resident_sources_hash(kernel_file: str = "sweep_resident.cu") -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for f in (kernel_file, "sweep_common.cuh", "philox.cuh"):
+    for f in (kernel_file, "sweep_common.cuh", "cluster_exchange.cuh", "philox.cuh"):
         with open(os.path.join(ROOT, "paper_1309_4349_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -481,7 +482,7 @@ def sub_c1(x):
                                  {"cluster": C, "threads_per_cta": T,
                                   "note": "one lattice of 4096 sites on one CTA: latency-bound"}),
            "clocks": clk, "gpu_launches": len(ms) * (LAUNCHES_SET_LATTICE_DEVICE +
-                                                    nseg * (LAUNCHES_SWEEP + LAUNCHES_HISTOGRAM))}
+                                                    nseg * (LAUNCHES_SWEEP + LAUNCHES_HISTOGRAM_SMALL))}
     lat.close()
     if not x.args.skip_cpu:
         import oracle
