@@ -80,7 +80,7 @@ ISSUE_LANES_PER_SM = 128
 # with (hash of the kernel's file + sweep_common.cuh + cluster_exchange.cuh + philox.cuh).
 TRAFFIC_C2_LAUNCH = 230656
 TRAFFIC_C3_LAUNCH = 8494336
-TRAFFIC_SOURCES = "6dd3276ed3228bd1"
+TRAFFIC_SOURCES = "650cc4995f465648"
 TRAFFIC_C6_LAUNCH = 93184
 TRAFFIC_HELICAL_SOURCES = "56a8f01e6f3bbf26"
 
@@ -480,7 +480,7 @@ def sub_c1(x):
            "roofline": _roofline("resident_sweep_kernel", launch_ms, attempts // nseg, cnt["draws"] / attempts,
                                  x.sm_count, _sm_mhz(clk), C, 2 * c["L"] * c["L"], x.l2_peak,
                                  {"cluster": C, "threads_per_cta": T,
-                                  "note": "one lattice of 4096 sites on one CTA: latency-bound"}),
+                                  "note": "one lattice of 4096 sites: latency-bound"}),
            "clocks": clk, "gpu_launches": len(ms) * (LAUNCHES_SET_LATTICE_DEVICE +
                                                     nseg * (LAUNCHES_SWEEP + LAUNCHES_HISTOGRAM_SMALL))}
     lat.close()

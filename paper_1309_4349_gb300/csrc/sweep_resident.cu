@@ -537,8 +537,8 @@ using Const = std::integral_constant<int, V>;
 // next kChunk phases while the others, which synchronise among themselves, run the
 // current ones, and meets them once per chunk.  (Two or four such warps were no faster,
 // and took warps from the tasks: 400^2 on 8 CTAs 1.55 us per phase with four, 1.39 with one.)
-// With 128 threads (several CTAs per SM, every warp busy) each of the four warps prepares one phase of the next chunk before
-// its own tasks.
+// With 128 threads (several CTAs per SM, every warp busy) each of the four warps
+// prepares one phase of the next chunk before its own tasks.
 template <int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB)
 resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__restrict__ calls,
@@ -759,10 +759,9 @@ constexpr int kBandThreads = KLMC_BAND_THREADS;  // one CTA per SM
 
 // Band kernel shared memory (32-bit words): rows (H + 2D) x RWb, the warps' draw
 // queues, then (where they fit) K task tables of W words (rounded up to even) and
-// 2 x rows words each.  A band row is the padded row of the resident kernel (word 0
-// holds position -1, words 1..W the sites, W+1 the last pads) placed 3 words into
-// RWb = W + 5 rounded up to 4 words, so that its sites start on a 16-byte boundary
-// and a row of the bit store lands there by one bulk copy.
+// 2 x rows words each.  A row's stride RWb is W + 5 words rounded up to 4, so that rows
+// start on 16-byte boundaries and a row of the bit store (at most W + 3 words) lands
+// there by one bulk copy.
 __host__ __device__ __forceinline__ int band_row_words(int W)
 {
     return (W + 5 + 3) / 4 * 4;
@@ -876,11 +875,10 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (bulk) {
-        // One bulk copy per row (pitch words, 16-byte aligned at both ends) into the
-        // row's site words, completing on one mbarrier whose expected byte count is
-        // exactly theirs; then the pad words.  Under the test hook no copy is
-        // issued and the barrier expects the hook's bytes instead, which nothing
-        // delivers: the wait runs out with no copy in flight.
+        // One bulk copy per row (pitch words, 16-byte aligned at both ends), completing
+        // on one mbarrier whose expected byte count is exactly theirs.  Under the test
+        // hook no copy is issued and the barrier expects the hook's bytes instead, which
+        // nothing delivers: the wait runs out with no copy in flight.
         __syncthreads();
         const bool hook = J.copy_shortfall != 0;
         if (tid < 32) {
@@ -1108,7 +1106,6 @@ cudaError_t launch_resident_sweep_one(const SweepJob &job, const SweepCall &call
 #ifndef KLMC_TILED_BLOCK
 #define KLMC_TILED_BLOCK 4
 #endif
-
 
 // Lattices that the automatic choice takes to the tiled path.
 constexpr long long kWideBlockSites = 786432;
