@@ -1,8 +1,10 @@
 // cluster_exchange.cuh -- the halo exchange of lattices resident in a thread-block
 // cluster's shared memory, between the CTAs of neighbouring bands.  Included inside
-// namespace klmc by the resident sweeps.
+// namespace klmc by the resident sweeps, and by tests/exchange_model.cpp, which runs
+// the exchange on the host over a model of the operations below.
 #pragma once
 
+#ifndef KLMC_EXCHANGE_MODEL
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -22,11 +24,30 @@ __device__ __forceinline__ uint32_t mapa_distance(uint32_t addr, int rank)
     return remote - addr;
 }
 
-// Polls of a wait before it gives up; once one has, the launch's other waits poll once.
-constexpr int kExchangePolls = 1 << 20;
+// Readies the mbarrier at shared address bar for one arrival per phase.
+__device__ __forceinline__ void mbar_init(uint32_t bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// The phase's one arrival; the phase completes with it and `bytes` of stores.
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
+{
+    unsigned long long st;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;" : "=l"(st) : "r"(bar), "r"(bytes) : "memory");
+}
+
+// Stores v at address `to` of another CTA of the cluster and counts its 4 bytes on the
+// mbarrier at address `bar` there.
+__device__ __forceinline__ void store_counted(uint32_t to, uint32_t v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                 ::"r"(to), "r"(v), "r"(bar) : "memory");
+}
 
 // Waits for phase `parity` of the mbarrier at shared address bar, which the stores of
-// another CTA of the cluster complete.
+// another CTA of the cluster complete; false after `limit` polls.
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int limit)
 {
     for (int i = 0; i < limit; ++i) {
@@ -40,21 +61,43 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
     return false;
 }
+#endif
 
-// What a CTA's block exchanges need: its two mbarriers (side 0: from the CTA above,
-// side 1: from the one below) and the distances from its own shared memory to theirs.
+// Polls of a wait before it gives up; once one has, the launch's other waits poll once.
+constexpr int kExchangePolls = 1 << 20;
+
+// A CTA's mbarriers: two sides (0: from the CTA above, 1: from the one below) of two
+// block parities.
+constexpr int kExchangeBars = 4;
+
+// What a CTA's block exchanges need: its mbarriers and the distances from its own
+// shared memory to its neighbours'.
 struct Exchange {
     uint32_t bar, to_prev, to_next;
     int polls;
     bool fault;
 };
 
+__device__ __forceinline__ uint32_t exchange_bar(uint32_t bar, uint32_t side, uint32_t parity)
+{
+    return bar + 16u * side + 8u * parity;
+}
+
 // End of a block: the D lowest and D highest band rows go to the mailboxes of parity
 // block & 1 in the neighbouring CTAs, by asynchronous stores that count their bytes on
 // the receiver's mbarriers; this CTA's own mailboxes then fill its halo rows.  A CTA
-// waits for its two neighbours only.  Two parities are enough: a neighbour's block
-// n + 2 follows its receipt of this CTA's n + 1, sent after n was read; and the two
-// sides count apart, because one neighbour may be a block ahead of the other.
+// waits for its two neighbours only.  The caller has a barrier of the NT threads before
+// and after.
+//
+// Nothing but the following orders the exchanges (a warp may stall anywhere, and
+// stores of one CTA may land in any order).  A neighbour sends block n + 2 after it
+// has received all of this CTA's block n + 1, which this CTA sends after its barrier
+// behind exchange n: by then every byte of block n has landed and been copied.  So
+// two mailboxes per side are enough, and two mbarriers: on the one of a side and parity
+// the bytes of block n + 2 come after the phase of block n is complete.  One mbarrier
+// per side would not do: a neighbour needs nothing of this CTA's first warp to be one
+// block ahead of it, and its block n + 1 would then count in the phase of block n.
+// Within a phase the arrival and the stores come in any order.
 // (With a cluster barrier instead, whose release waits for the stores to be
 // acknowledged, an exchange took about 0.8 us of a 400^2 lattice on 16 CTAs.)
 template <int NT>
@@ -62,24 +105,19 @@ __device__ __forceinline__ void exchange_halos(uint32_t *lat, uint32_t lat_addr,
                                                Exchange &X)
 {
     const int rw = D * RW;
-    const uint32_t p = (uint32_t)block & 1u;
+    const uint32_t p = (uint32_t)block & 1u, phase = ((uint32_t)block >> 1) & 1u;
     uint32_t *const mbox = lat + (hmax + 2 * D) * RW + 2 * p * rw;
     const uint32_t mbox_addr = lat_addr + 4u * (uint32_t)((hmax + 2 * D) * RW + 2 * p * rw);
-    if (threadIdx.x < 2) {
-        unsigned long long st;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;"
-                     : "=l"(st) : "r"(X.bar + 8u * threadIdx.x), "r"(4u * (uint32_t)rw) : "memory");
-    }
+    if (threadIdx.x < 2) mbar_expect(exchange_bar(X.bar, threadIdx.x, p), 4u * (uint32_t)rw);
     for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
         const bool low = idx >= rw;  // the lowest rows go up (side 1 there), the highest down (side 0)
         const uint32_t v = lat[low ? D * RW + idx - rw : H * RW + idx];
         const uint32_t to = low ? X.to_prev : X.to_next;
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                     ::"r"(mbox_addr + 4u * (uint32_t)idx + to), "r"(v), "r"(X.bar + (low ? 8u : 0u) + to) : "memory");
+        store_counted(mbox_addr + 4u * (uint32_t)idx + to, v, exchange_bar(X.bar, low ? 1u : 0u, p) + to);
     }
     for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
         const bool low = idx >= rw;
-        if (!mbar_wait_cluster(X.bar + (low ? 8u : 0u), p, X.polls)) {
+        if (!mbar_wait_cluster(exchange_bar(X.bar, low ? 1u : 0u, p), phase, X.polls)) {
             X.polls = 1;
             X.fault = true;
         }
@@ -87,13 +125,10 @@ __device__ __forceinline__ void exchange_halos(uint32_t *lat, uint32_t lat_addr,
     }
 }
 
-// Readies the two mbarriers (before the cluster barrier that precedes the first exchange).
+// Readies the mbarriers (before the cluster barrier that precedes the first exchange).
 __device__ __forceinline__ void exchange_init(unsigned long long *xbar)
 {
-    if (threadIdx.x < 2) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(xbar + threadIdx.x)) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (threadIdx.x < kExchangeBars) mbar_init(smem_addr(xbar + threadIdx.x));
 }
 
 __device__ __forceinline__ Exchange exchange_for(const unsigned long long *xbar, uint32_t lat_addr, int C, int rank)
@@ -109,8 +144,8 @@ __device__ __forceinline__ void exchange_end(const Exchange &X, long long *state
 {
     if (__syncthreads_or(X.fault)) {
         if (threadIdx.x == 0) atomicExch((unsigned long long *)&state[kFault], 1ull);
-        for (int side = 0; side < 2; ++side)
-            for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * side, par, kExchangePolls);
+        for (uint32_t i = 0; i < kExchangeBars; ++i)
+            for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * i, par, kExchangePolls);
     }
     cluster_barrier();
 }

@@ -221,7 +221,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     extern __shared__ __align__(16) uint32_t lat[];
     __shared__ long long red[5][kWarps];
     __shared__ HSched sched[2];  // the current and the next iteration
-    __shared__ __align__(8) unsigned long long xbar[2];
+    __shared__ __align__(8) unsigned long long xbar[kExchangeBars];
     if (Cl.n_mcs <= 0) return;
 
     HGeo g;

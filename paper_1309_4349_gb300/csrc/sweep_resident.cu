@@ -553,7 +553,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     __shared__ PhaseR pp[2][kChunk];
     __shared__ PhaseHdr hdr[2][kChunk];
     __shared__ long long red[5][kWarps];
-    __shared__ __align__(8) unsigned long long xbar[2];
+    __shared__ __align__(8) unsigned long long xbar[kExchangeBars];
 
     const int C = (int)cluster_nctarank();
     const int rank = (int)cluster_ctarank();
