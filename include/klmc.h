@@ -262,7 +262,8 @@ klmc_status klmc_get_counters(klmc_ctx *c, klmc_counters *out);
  * tiled launch of this handle that moves its rows by bulk copies issues no row
  * copy and waits instead for `bytes` that nothing delivers, so that its wait gives
  * up after a short bound with no copy in flight; the launch then leaves its band
- * unwritten and klmc_energy /
+ * unwritten.  A resident launch whose CTAs exchange rows sends none and waits for
+ * them as briefly (bytes only switches it on).  Either way klmc_energy /
  * klmc_get_counters report KLMC_ETIMEOUT.  The handle's lattice is then no longer
  * a state of the chain; other handles are unaffected.  Synchronises.  EINVAL for
  * bytes < 0. */

@@ -352,8 +352,8 @@ class Lattice:
         return c.as_dict()
 
     def test_copy_shortfall(self, nbytes: int):
-        """Test hook: make this handle's tiled launches wait for row copies that
-        never arrive (klmc_test_copy_shortfall)."""
+        """Test hook: make this handle's launches wait for rows that never arrive
+        (klmc_test_copy_shortfall)."""
         _check(lib().klmc_test_copy_shortfall(self._h, int(nbytes)))
 
     def get_lattice(self) -> np.ndarray:

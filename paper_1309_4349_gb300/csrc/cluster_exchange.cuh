@@ -63,19 +63,22 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
 }
 #endif
 
-// Polls of a wait before it gives up; once one has, the launch's other waits poll once.
+// Polls of a wait before it gives up, and under the test hook (SweepJob::copy_shortfall).
 constexpr int kExchangePolls = 1 << 20;
+constexpr int kExchangePollsShort = 1 << 12;
 
 // A CTA's mbarriers: two sides (0: from the CTA above, 1: from the one below) of two
 // block parities.
 constexpr int kExchangeBars = 4;
 
-// What a CTA's block exchanges need: its mbarriers and the distances from its own
-// shared memory to its neighbours'.
+// What a thread's part in its CTA's exchanges needs: the CTA's mbarriers, the distances
+// from its own shared memory to its neighbours', the polls of a wait (kExchangePollsShort:
+// the test hook, under which no store is sent; 0: a wait of this thread ran out, and it
+// takes no further part), and the sides whose mbarriers the thread arms (bits 0 and 1).
 struct Exchange {
     uint32_t bar, to_prev, to_next;
     int polls;
-    bool fault;
+    uint32_t arms;
 };
 
 __device__ __forceinline__ uint32_t exchange_bar(uint32_t bar, uint32_t side, uint32_t parity)
@@ -98,6 +101,13 @@ __device__ __forceinline__ uint32_t exchange_bar(uint32_t bar, uint32_t side, ui
 // per side would not do: a neighbour needs nothing of this CTA's first warp to be one
 // block ahead of it, and its block n + 1 would then count in the phase of block n.
 // Within a phase the arrival and the stores come in any order.
+//
+// A thread whose wait ran out takes no further part, and the side's mbarrier is armed by
+// a thread that waits on it: so no arrival meets a phase that still lacks its bytes.  The
+// waits for what that thread does not send run out in turn, a CTA further with every
+// block, so that a barrier left behind takes the bytes of at most as many blocks as the
+// cluster has CTAs (16 x 33 KB, as a band is no lower than its halo; the count holds
+// 2^20 - 1).
 // (With a cluster barrier instead, whose release waits for the stores to be
 // acknowledged, an exchange took about 0.8 us of a 400^2 lattice on 16 CTAs.)
 template <int NT>
@@ -108,18 +118,23 @@ __device__ __forceinline__ void exchange_halos(uint32_t *lat, uint32_t lat_addr,
     const uint32_t p = (uint32_t)block & 1u, phase = ((uint32_t)block >> 1) & 1u;
     uint32_t *const mbox = lat + (hmax + 2 * D) * RW + 2 * p * rw;
     const uint32_t mbox_addr = lat_addr + 4u * (uint32_t)((hmax + 2 * D) * RW + 2 * p * rw);
-    if (threadIdx.x < 2) mbar_expect(exchange_bar(X.bar, threadIdx.x, p), 4u * (uint32_t)rw);
+    if (X.arms != 0u) {
+        if (X.arms & 1u) mbar_expect(exchange_bar(X.bar, 0u, p), 4u * (uint32_t)rw);
+        if (X.arms & 2u) mbar_expect(exchange_bar(X.bar, 1u, p), 4u * (uint32_t)rw);
+    }
     for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
         const bool low = idx >= rw;  // the lowest rows go up (side 1 there), the highest down (side 0)
         const uint32_t v = lat[low ? D * RW + idx - rw : H * RW + idx];
         const uint32_t to = low ? X.to_prev : X.to_next;
-        store_counted(mbox_addr + 4u * (uint32_t)idx + to, v, exchange_bar(X.bar, low ? 1u : 0u, p) + to);
+        if (X.polls == kExchangePolls)
+            store_counted(mbox_addr + 4u * (uint32_t)idx + to, v, exchange_bar(X.bar, low ? 1u : 0u, p) + to);
     }
     for (int idx = threadIdx.x; idx < 2 * rw; idx += NT) {
         const bool low = idx >= rw;
         if (!mbar_wait_cluster(exchange_bar(X.bar, low ? 1u : 0u, p), phase, X.polls)) {
-            X.polls = 1;
-            X.fault = true;
+            X.polls = 0;
+            X.arms = 0u;
+            break;
         }
         lat[low ? (D + H) * RW + idx - rw : idx] = mbox[idx];
     }
@@ -131,21 +146,27 @@ __device__ __forceinline__ void exchange_init(unsigned long long *xbar)
     if (threadIdx.x < kExchangeBars) mbar_init(smem_addr(xbar + threadIdx.x));
 }
 
-__device__ __forceinline__ Exchange exchange_for(const unsigned long long *xbar, uint32_t lat_addr, int C, int rank)
+// halo_words: D * RW.  Side 0 is armed by the thread of the first word of a halo, side 1
+// by that of the first word from below: the first that each waits for.
+template <int NT>
+__device__ __forceinline__ Exchange exchange_for(const unsigned long long *xbar, uint32_t lat_addr, int C, int rank,
+                                                 int halo_words, bool withhold)
 {
     return {smem_addr(xbar), mapa_distance(lat_addr, rank == 0 ? C - 1 : rank - 1),
-            mapa_distance(lat_addr, rank + 1 == C ? 0 : rank + 1), kExchangePolls, false};
+            mapa_distance(lat_addr, rank + 1 == C ? 0 : rank + 1), withhold ? kExchangePollsShort : kExchangePolls,
+            (threadIdx.x == 0 ? 1u : 0u) | ((int)threadIdx.x == halo_words % NT ? 2u : 0u)};
 }
 
 // By every thread after the last exchange.  A wait that ran out leaves a lattice that is no
 // state of the chain: report it, and give stores in flight a second bounded wait.  No CTA
 // leaves while a peer may still write into it.
-__device__ __forceinline__ void exchange_end(const Exchange &X, long long *state)
+__device__ __forceinline__ void exchange_end(const Exchange &X, bool withhold, long long *state)
 {
-    if (__syncthreads_or(X.fault)) {
+    if (__syncthreads_or(X.polls == 0)) {
         if (threadIdx.x == 0) atomicExch((unsigned long long *)&state[kFault], 1ull);
+        const int polls = withhold ? kExchangePollsShort : kExchangePolls;
         for (uint32_t i = 0; i < kExchangeBars; ++i)
-            for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * i, par, kExchangePolls);
+            for (uint32_t par = 0; par < 2; ++par) mbar_wait_cluster(X.bar + 8u * i, par, polls);
     }
     cluster_barrier();
 }

@@ -43,7 +43,8 @@ struct SweepJob {
     int32_t draw_lo;      // neighbour-agreement sums S in [draw_lo, draw_hi] need a draw
     int32_t draw_hi;
     int32_t copy_shortfall;  // test hook (0 in use): a band launch issues no row copy and waits for
-                             // this many bytes instead, which nothing delivers, so its bounded wait runs out
+                             // this many bytes instead, which nothing delivers, so its bounded wait runs out;
+                             // a cluster's CTAs withhold their exchanges' stores
     uint64_t thr[16];     // accept iff draw < thr[S] (S = same_a + same_b)
     // The same table as the kernels read it: a draw r of a pair of class c (the two low bits
     // of its S, see sweep_common.cuh) is accepted iff r <= draw_t[c], or never when bit c

@@ -264,7 +264,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
     long long t_dn = 0;
     int jb = 0, pb = 0;  // iteration within the block; buffer of the current schedule entry
     int block = 0;
-    Exchange X = exchange_for(xbar, g.lat_addr, g.C, g.rank);
+    Exchange X = exchange_for<kHelicalThreads>(xbar, g.lat_addr, g.C, g.rank, g.D * g.RW, J.copy_shortfall != 0);
     const HWord word = helical_word(g, tid);
     for (long long it = 0; it < Cl.n_mcs; ++it) {
         const unsigned long long s = (unsigned long long)(Cl.sweep0 + it);
@@ -308,7 +308,7 @@ helical_resident_kernel(const SweepJob J, const SweepCall Cl)
         }
     }
 
-    exchange_end(X, J.state);
+    exchange_end(X, J.copy_shortfall != 0, J.state);
 
     // Write the band back (sites only).
     for (int idx = tid; idx < g.H * g.W; idx += kHelicalThreads) {

@@ -643,7 +643,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
     // The preparing warps: the next chunk's tables while the current one runs, then the
     // chunk's last barrier (every phase is a cluster barrier when bands are too thin
     // for blocks).
-    Exchange X = exchange_for(xbar, g.lat_addr, C, rank);
+    Exchange X = exchange_for<NT>(xbar, g.lat_addr, C, rank, g.D * g.RW, J.copy_shortfall != 0);
     auto run_tasks = [&](auto geometry, auto is_blocked, auto has_fix) {
         constexpr int G = decltype(geometry)::value;
         constexpr bool BLOCKED = decltype(is_blocked)::value;
@@ -727,7 +727,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         if (g.tri) run_tasks(Const<kTRI6>{}, std::false_type{}, std::true_type{});
         else run_tasks(Const<kSQ4>{}, std::false_type{}, std::true_type{});
     }
-    if (blocked) exchange_end(X, J.state);
+    if (blocked) exchange_end(X, J.copy_shortfall != 0, J.state);
 
     // Write the band back (main positions only).
     for (int idx = tid; idx < H * g.W; idx += THREADS) {

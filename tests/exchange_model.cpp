@@ -4,7 +4,8 @@
 // PTX ISA defines them.  Adversaries hold back a warp or single stores for as long as
 // anything else can move.  After every exchange each CTA's halo rows must be its
 // neighbours' rows of that block, no wait may run out, and no arrival may meet a phase that
-// has had its one.
+// has had its one.  When a store is lost, waits run out: the cluster must come to its end
+// all the same, report it, and stay within the rules of the mbarriers.
 #include <ucontext.h>
 
 #include <cstdint>
@@ -40,14 +41,14 @@ struct Message {
 struct Cta {
     std::vector<uint32_t> smem;
     long long state[16] = {};
-    int waiting = 0, generation = 0, vote = 0, voted = 0;
+    int waiting = 0, generation = 0, vote = 0;
 };
 
 struct Fiber {
     ucontext_t uc;
     std::vector<char> stack;
     int cta = 0, tid = 0;
-    bool done = false, gave_up = false;
+    bool done = false, gave_up = false, polling = false;
     std::function<bool()> ready;  // empty: may run
 };
 
@@ -59,6 +60,7 @@ Fiber *self = nullptr;
 ucontext_t scheduler;
 int threads = 0, cluster_waiting = 0, cluster_generation = 0;
 long sent = 0, timeouts = 0, faults_found = 0;
+bool rows_matter = true, withhold = false;
 struct { unsigned x; } threadIdx;
 
 void found(const char *what)
@@ -120,11 +122,11 @@ void store_counted(uint32_t to, uint32_t v, uint32_t bar)
 
 bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int)
 {
-    if (!pause_until([=] { return (bars.at(bar).phase & 1u) != parity; })) {
-        timeouts += 1;
-        return false;
-    }
-    return true;
+    self->polling = true;
+    const bool ok = pause_until([=] { return (bars.at(bar).phase & 1u) != parity; });
+    self->polling = false;
+    if (!ok) timeouts += 1;
+    return ok;
 }
 
 void cta_barrier()
@@ -153,11 +155,7 @@ int __syncthreads_or(int v)
     Cta &c = ctas[self->cta];
     c.vote |= v;
     cta_barrier();
-    const int r = c.vote;
-    cta_barrier();
-    c.vote = 0;
-    cta_barrier();
-    return r;
+    return c.vote;  // (one call in a run)
 }
 
 unsigned long long atomicExch(unsigned long long *p, unsigned long long v)
@@ -186,7 +184,7 @@ void thread_main(const Shape &s)
     uint32_t *const lat = cta.smem.data() + 16;
     exchange_init(xbar);
     cluster_barrier();
-    Exchange X = exchange_for(xbar, smem_addr(lat), s.C, c);
+    Exchange X = exchange_for<NT>(xbar, smem_addr(lat), s.C, c, s.D * s.RW, withhold);
     const int prev = (c + s.C - 1) % s.C, next = (c + 1) % s.C;
     for (int b = 0; b < s.blocks; ++b) {
         for (int i = self->tid; i < s.H * s.RW; i += NT) lat[s.D * s.RW + i] = site(c, i / s.RW, i % s.RW, b);
@@ -195,12 +193,13 @@ void thread_main(const Shape &s)
         cta_barrier();
         for (int i = self->tid; i < s.D * s.RW; i += NT) {
             const int r = i / s.RW, w = i % s.RW;
+            if (!rows_matter) continue;
             if (lat[i] != site(prev, s.H - s.D + r, w, b)) found("a halo row that is not the upper neighbour's");
             if (lat[(s.D + s.H + r) * s.RW + w] != site(next, r, w, b)) found("a halo row that is not the lower neighbour's");
         }
         cta_barrier();
     }
-    exchange_end(X, cta.state);
+    exchange_end(X, withhold, cta.state);
 }
 
 template <int NT>
@@ -213,11 +212,16 @@ void fiber_main(unsigned lo, unsigned hi)
 
 enum Order { kAny, kOldestStore, kNewestStore };
 
+// What becomes of the held stores when nothing else can move: they land, never do, or do
+// after a wait or more has run out.
+enum Held { kLate, kLost, kTooLate };
+
 // Runs the cluster under one adversary; true when all went well.
 template <int NT>
 bool run(const Shape &s, std::function<bool(const Fiber &)> held_fiber, std::function<bool(const Message &)> held_store,
-         Order order, unsigned seed)
+         Order order, unsigned seed, Held fate = kLate)
 {
+    rows_matter = fate == kLate;
     ctas.assign(s.C, Cta());
     bars.clear();
     flying.clear();
@@ -272,24 +276,27 @@ bool run(const Shape &s, std::function<bool(const Fiber &)> held_fiber, std::fun
             step(free[rng() % free.size()]);
         } else if (!held.empty()) {
             step(held[rng() % held.size()]);
-        } else if (!held_stores.empty()) {
+        } else if (!held_stores.empty() && (fate == kLate || (fate == kTooLate && timeouts > 0 && rng() % 4 == 0))) {
             land(held_stores[rng() % held_stores.size()]);
-        } else {  // nothing can move: the waits run out
-            Fiber *w = nullptr;
+        } else {  // nothing can move: a wait runs out
+            std::vector<Fiber *> polling;
             for (auto &f : fibers)
-                if (!f->done && !w) w = f.get();
-            for (auto &f : fibers)
-                if (!f->done && f->ready && rng() % 8 == 0) w = f.get();
-            w->gave_up = true;
-            step(w);
-            if (timeouts == 0) found("threads that wait at a barrier for ever");
-            if (timeouts > 0 && faults_found == 0) found("a wait that nothing ends");
-            return false;
+                if (!f->done && f->polling) polling.push_back(f.get());
+            if (polling.empty()) {
+                found("threads that wait at a barrier for ever");
+                return false;
+            }
+            Fiber *const f = polling[rng() % polling.size()];
+            f->gave_up = true;
+            step(f);
         }
     }
-    for (Cta &c : ctas)
-        if (c.state[kFault] != 0) found("a reported fault");
-    return faults_found == 0 && timeouts == 0;
+    int reports = 0;
+    for (Cta &c : ctas) reports += c.state[kFault] != 0;
+    if (fate == kLate && (timeouts > 0 || reports > 0)) found("a wait that nothing ends");
+    if (withhold && (sent > 0 || reports < s.C)) found("stores sent, or a CTA without a report, under the test hook");
+    if (fate != kLate && (timeouts == 0 || reports == 0)) found("a wait that ran out and nobody reports");
+    return faults_found == 0;
 }
 
 int failures = 0;
@@ -312,12 +319,21 @@ void all_adversaries(const Shape &s)
         for (int w = 0; w < NT / 32; ++w)
             check(run<NT>(s, [=](const Fiber &f) { return f.cta == c && f.tid / 32 == w; }, nullptr, kOldestStore, 7),
                   "a warp held back: CTA, warp", s, NT, c, w);
+    withhold = true;
+    check(run<NT>(s, nullptr, nullptr, kAny, 0, kLost), "stores withheld", s, NT, 0, 0);
+    withhold = false;
     const long all = (long)s.C * s.blocks * 2 * s.D * s.RW;
     std::mt19937 rng(11);
     for (int k = 0; k < 12; ++k) {
         const long n = (long)(rng() % (unsigned long)all);
         check(run<NT>(s, nullptr, [=](const Message &m) { return m.number == n; }, kOldestStore, (unsigned)k),
               "a store held back: number", s, NT, (int)n, 0);
+        const long few = n % (2l * s.C * 2 * s.D * s.RW);  // of the first two blocks
+        check(run<NT>(s, nullptr, [=](const Message &m) { return m.number == few; }, kOldestStore, (unsigned)k, kLost),
+              "a store lost: number", s, NT, (int)few, 0);
+        check(run<NT>(s, nullptr, [=](const Message &m) { return m.number >= few && m.number < few + 40; }, kAny, (unsigned)k,
+                      kTooLate),
+              "stores too late: from number", s, NT, (int)few, 0);
     }
 }
 
