@@ -428,7 +428,9 @@ klmc_status klmc_server_create(klmc_server **out, size_t device_mem_budget, void
 klmc_status klmc_server_submit(klmc_server *s, const klmc_params *p, int64_t n_mcs,
                                int64_t hist_every, uint32_t flags, uint64_t *job_id);
 
-/* Result of a job; KLMC_EBUSY while it is queued or running. */
+/* Result of a job; KLMC_EBUSY while it is queued or running.  A job one of whose
+ * launches gave up a bounded wait (see klmc_energy) has status KLMC_ETIMEOUT and
+ * leaves neither histogram nor lattice. */
 klmc_status klmc_server_poll(klmc_server *s, uint64_t job_id, klmc_job_result *out);
 
 /* Final lattice (one byte per site) of a finished job submitted with

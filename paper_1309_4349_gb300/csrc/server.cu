@@ -353,7 +353,9 @@ klmc_status run_round(klmc_server *s)
     s->rounds += 1;
     for (Job *j : finishing) {
         e = cudaMemcpy(j->final_state, j->ctx->state, sizeof(j->final_state), cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess && j->dhist) {
+        // A launch of the job gave up a bounded wait: what it holds is no result.
+        const bool gave_up = e == cudaSuccess && j->final_state[klmc::kFault] != 0;
+        if (e == cudaSuccess && !gave_up && j->dhist) {
             long long nd = 0;
             e = cudaMemcpy(&nd, j->dhist + 2 * j->hist_cap, sizeof(nd), cudaMemcpyDeviceToHost);
             if (e == cudaSuccess && nd > 0 && nd <= j->hist_cap) {
@@ -365,14 +367,14 @@ klmc_status run_round(klmc_server *s)
                                    cudaMemcpyDeviceToHost);
             }
         }
-        if (e == cudaSuccess && (j->flags & KLMC_JOB_KEEP_LATTICE)) {
+        if (e == cudaSuccess && !gave_up && (j->flags & KLMC_JOB_KEEP_LATTICE)) {
             j->lattice.resize((size_t)j->ctx->N);
             klmc_status ls = klmc_get_lattice(j->ctx, j->lattice.data(), j->ctx->N);
             if (ls != KLMC_OK) e = cudaErrorUnknown;
         }
         std::lock_guard<std::mutex> lock(s->mu);
-        s->attempts += j->final_state[klmc::kAttempts];
-        retire(s, j, e == cudaSuccess ? KLMC_OK : KLMC_ECUDA);
+        if (!gave_up) s->attempts += j->final_state[klmc::kAttempts];
+        retire(s, j, e != cudaSuccess ? KLMC_ECUDA : (gave_up ? KLMC_ETIMEOUT : KLMC_OK));
         s->done_cv.notify_all();
     }
     if (!finishing.empty()) {
