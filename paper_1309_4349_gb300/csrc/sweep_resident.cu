@@ -470,6 +470,8 @@ constexpr int kResidentMaxSmem = 227 * 1024 - 6144;
 #ifndef KLMC_MAX_BLOCK
 #define KLMC_MAX_BLOCK 4
 #endif
+static_assert(KLMC_MAX_BLOCK == 1 || KLMC_MAX_BLOCK == 2 || KLMC_MAX_BLOCK == 4 || KLMC_MAX_BLOCK == 8,
+              "a sweep's 8 phases are whole blocks");
 
 // Phases per block for a lattice of Lx x Ly sites split over C CTAs: the largest K
 // of 8, 4, 2 (at most KLMC_MAX_BLOCK) whose halo D = 2K + 1 fits in every band
@@ -681,8 +683,10 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
                         cluster_barrier();
                         continue;
                     }
-                    // Blocks of K phases end with an exchange, except the launch's last.
-                    if (BLOCKED && ((q + 1) & (K - 1)) == 0 && !(last && buf == 1 && q == kChunk - 1)) {
+                    // Blocks of K phases end with an exchange, except the launch's last.  (One of
+                    // more than kChunk phases ends in a later chunk than it began.)
+                    const int ran = (KLMC_MAX_BLOCK > kChunk ? kChunk * buf : 0) + q + 1;
+                    if (BLOCKED && (ran & (K - 1)) == 0 && !(last && buf == 1 && q == kChunk - 1)) {
                         task_barrier<NT>();
                         exchange_halos<NT>(lat, g.lat_addr, g.RW, g.Y1 - g.Y0, g.D, hmax, block++, X);
                     }
