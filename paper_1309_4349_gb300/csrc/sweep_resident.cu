@@ -173,12 +173,11 @@ __device__ __forceinline__ bool table_fits(const Geo &g, const PhaseR &P, const 
 }
 
 // Fills the table entries with index = lane0 mod step, so that a warp (step 32) or a
-// CTA (step THREADS) builds it together.
+// CTA (step THREADS) builds it together.  The table holds the phase's words and rows.
 template <bool BLOCKED>
 __device__ __forceinline__ void build_task_table(const PhaseR &P, const Geo &g, const TaskTab &T, int lane0,
                                                  int step)
 {
-    if (!table_fits(g, P, T)) return;
     for (int j = lane0; j < g.W; j += step) T.am[j] = anchor_mask(j << 5, P, g.Lx);
     for (int mi = lane0; mi < P.c[3]; mi += step) {
         const int m = mi < P.c[0] ? P.a[0] + mi
@@ -500,10 +499,12 @@ __device__ __forceinline__ void phase_table(const Geo &g, int K, long long s, in
 }
 
 // Words of the task tables of one phase, and of the two chunks' (see TaskTab): anchor
-// masks of W words (even, so that the row entries stay aligned) and the rows.
+// masks of W words (even, so that the row entries stay aligned) and the rows.  They hold
+// every phase: its anchor rows lie in at most hmax + 2 (2K - 1) rows (K = 1: hmax) and are
+// at least two apart, around the lattice's end too, so there are at most (hmax + 4K) / 2.
 __host__ __device__ __forceinline__ int phase_table_words(int W, int hmax, int K)
 {
-    return ((W + 1) & ~1) + 2 * ((hmax + 4 * K) / 2 + 2);  // anchor rows of hmax + 2(2K - 1) rows, 2 apart
+    return ((W + 1) & ~1) + 2 * ((hmax + 4 * K) / 2 + 2);
 }
 __host__ __device__ __forceinline__ long long chunk_table_words(int W, int hmax, int K)
 {
@@ -629,7 +630,7 @@ resident_sweep_kernel(const SweepJob *__restrict__ jobs, const SweepCall *__rest
         for (int q = q0; q < q0 + kPer; ++q) {
             const PhaseR P = pp[buf][q];
             uint32_t *const t = tab_base + (buf * kChunk + q) * tab_words;
-            const TaskTab tt = {t, (int2 *)(t + g.tabW), g.W, tab_words};
+            const TaskTab tt = {t, (int2 *)(t + g.tabW), g.W, (tab_words - g.tabW) / 2};
             if (blocked) build_task_table<true>(P, g, tt, lane, 32);
             else build_task_table<false>(P, g, tt, lane, 32);
         }
@@ -868,7 +869,7 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
             const PhaseR P = pp[q];
             uint32_t *const t = tab_base + (size_t)q * (tab_w + 2 * tab_rows);
             const TaskTab T = {t, (int2 *)(t + tab_w), g.W, tab_rows};
-            build_task_table<true>(P, g, T, tid, THREADS);
+            if (table_fits(g, P, T)) build_task_table<true>(P, g, T, tid, THREADS);
         }
     }
     // the warps' draw queues follow the rows (H + 2D rows of the tallest band)
