@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -959,12 +960,12 @@ klmc_status klmc_cluster_histogram(klmc_ctx *c, int32_t species, int64_t *sizes,
                                        (int64_t *)dn);
     if (st != KLMC_OK) return st;
     // Small lattices' whole output block in one copy: one wait instead of two (64^2: 61 -> 45 us).
+    // Without host memory for it, as for larger ones (no exception may leave a C entry).
     const size_t total = (size_t)(2 * c->hist_cap + 1);
-    std::vector<long long> block;
+    std::unique_ptr<long long[]> block(total * 8 <= 65536 ? new (std::nothrow) long long[total] : nullptr);
     long long n = 0;
-    if (total * 8 <= 65536) {
-        block.resize(total);
-        KLMC_CUDA(cudaMemcpyAsync(block.data(), dsz, total * 8, cudaMemcpyDeviceToHost, c->stream));
+    if (block) {
+        KLMC_CUDA(cudaMemcpyAsync(block.get(), dsz, total * 8, cudaMemcpyDeviceToHost, c->stream));
         KLMC_CUDA(cudaStreamSynchronize(c->stream));
         n = block[total - 1];
     } else {
@@ -976,9 +977,9 @@ klmc_status klmc_cluster_histogram(klmc_ctx *c, int32_t species, int64_t *sizes,
         *n_distinct = n;
         return fail(KLMC_ETRUNC, "capacity " + std::to_string(capacity) + " < " + std::to_string(n));
     }
-    if (!block.empty()) {
-        std::copy_n(block.begin(), n, sizes);
-        std::copy_n(block.begin() + c->hist_cap, n, counts);
+    if (block) {
+        std::copy_n(block.get(), n, sizes);
+        std::copy_n(block.get() + c->hist_cap, n, counts);
     } else if (n > 0) {
         KLMC_CUDA(cudaMemcpyAsync(sizes, dsz, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream));
         KLMC_CUDA(cudaMemcpyAsync(counts, dct, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream));
