@@ -28,13 +28,17 @@ namespace {
 
 constexpr int kTileRows = 32, kTileWords = 8;
 constexpr int kTileThreads = kTileRows * kTileWords;         // one per word
-constexpr int kTileSites = 32 * kTileThreads;
+// Places of a word's sites in the trees: 33, so that one place of all the words of a warp
+// lies in 32 banks.  (With 32, all of a column lay in one: columns of single sites, 256 x
+// 128, 173 -> 117 us; disordered lattices the same.)
+constexpr int kPlaces = 33;
+constexpr int kTilePlaces = kPlaces * kTileThreads;
 constexpr int kSmallSizes = 256;                             // sizes counted in shared memory first
 constexpr int kSmallMaxThreads = 1024;  // words of a lattice that one CTA holds
 constexpr int kCountThreads = 512;
-constexpr int kTileSmem = kTileSites * (4 + 2);
-// per word of a small lattice: 32 places (33 as a histogram, spread over the banks), counts, bits
-constexpr int kSmallWordSmem = 33 * 4 + 32 * 2 + 4;
+constexpr int kTileSmem = kTilePlaces * (4 + 2);
+// per word of a small lattice: places (then a histogram), counts (a pair of places each), bits
+constexpr int kSmallWordSmem = kPlaces * 4 + (kPlaces + 1) * 2 + 4;
 
 struct CcJob {
     const void *lat;
@@ -164,8 +168,8 @@ __device__ __forceinline__ TileLabels tile_labels(const CcJob &J, const ClusterS
 __global__ void __launch_bounds__(kTileThreads, 4)
 cc_tiles_kernel(const CcJob J, const ClusterScratch s, int tiles)
 {
-    extern __shared__ __align__(16) int32_t parent[];  // a place per site, then the counts
-    uint32_t *const cnt = (uint32_t *)(parent + kTileSites);
+    extern __shared__ __align__(16) int32_t parent[];  // the places, then the counts
+    uint32_t *const cnt = (uint32_t *)(parent + kTilePlaces);
     __shared__ uint32_t bits[kTileRows + 1][kTileWords + 2];  // row and word + 1; zeros around
     __shared__ int small[kSmallSizes];
     __shared__ int nodes;
@@ -182,17 +186,16 @@ cc_tiles_kernel(const CcJob J, const ClusterScratch s, int tiles)
         const uint32_t v = in ? species_word(J, y, gw) : 0u;
         bits[r][w + 1] = v;
         if (tid == 0) nodes = 0;
-        const int base = 32 * tid;
-        for (int i = 0; i < 8; ++i) {  // every site its own root, nothing counted
-            const int k = 4 * (tid + i * kTileThreads);
+        const int base = kPlaces * tid;
+        for (int k = 4 * tid; k < kTilePlaces; k += 4 * kTileThreads) {  // every site its own root, nothing counted
             *(int4 *)(parent + k) = make_int4(k, k + 1, k + 2, k + 3);
-            if (i < 4) *(int4 *)(cnt + k) = make_int4(0, 0, 0, 0);
+            if (k < kTilePlaces / 2) *(int4 *)(cnt + k) = make_int4(0, 0, 0, 0);
         }
         __syncthreads();
         {
             const uint32_t right = bits[r][w + 2], vleft = bits[r][w], b = bits[r + 1][w + 1], bleft = bits[r + 1][w];
-            if ((v >> 31) & right & 1u) unite(parent, base + run_start(v, 31), base + 32);
-            const int below = base + 32 * kTileWords;
+            if ((v >> 31) & right & 1u) unite(parent, base + run_start(v, 31), base + kPlaces);
+            const int below = base + kPlaces * kTileWords;
             for (uint32_t m = straight_contacts(v, b); m != 0u; m &= m - 1u) {
                 const int p = __ffs(m) - 1;
                 unite(parent, base + run_start(v, p), below + run_start(b, p));
@@ -202,7 +205,7 @@ cc_tiles_kernel(const CcJob J, const ClusterScratch s, int tiles)
                      m &= m - 1u) {
                     const int p = __ffs(m) - 1;
                     unite(parent, base + run_start(v, p),
-                          p > 0 ? below + run_start(b, p - 1) : below - 32 + run_start(bleft, 31));
+                          p > 0 ? below + run_start(b, p - 1) : below - kPlaces + run_start(bleft, 31));
                 }
             }
         }
@@ -257,23 +260,29 @@ cc_tiles_kernel(const CcJob J, const ClusterScratch s, int tiles)
         if (small[i] != 0) count_size(s, i, small[i]);
 }
 
-// Unions across tile borders.  Items 0 .. trows W - 1: a word of a tile row's last row
-// against the row below it; then tcols Ly items: a row at the right end of a tile column
+// Unions across tile borders.  Items 0 .. kParts trows W - 1: a part of a word of a tile
+// row's last row against the row below it (a union is a chain of waits for memory, and an
+// ordered lattice has 16 a word; 400^2, columns of single sites, with whole words 186 us,
+// in 8 parts 91, in 16 parts 85 but 8192^2 demixed slower); then tcols Ly items: a row at the right end of a tile column
 // against the first site of the next.  Around the lattice's sides the x wrap stays in
 // its row (periodic) or carries into the next or previous row (helical).
+constexpr int kParts = 8;
+
 __global__ void cc_merge_kernel(const CcJob J, const ClusterScratch s, long long items)
 {
     const int nlast = J.Lx - 32 * (J.W - 1);
     for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < items;
          it += (long long)gridDim.x * blockDim.x) {
-        if (it < (long long)J.trows * J.W) {
-            const int tr = (int)(it / J.W), w = (int)(it - (long long)tr * J.W);
+        const long long words = (long long)J.trows * J.W;
+        if (it < kParts * words) {
+            const int tr = (int)(it / kParts / J.W), w = (int)(it / kParts - (long long)tr * J.W);
+            const uint32_t part = (0xFFFFFFFFu >> (32 - 32 / kParts)) << (32 / kParts * (int)(it % kParts));
             const int y = min((tr + 1) * kTileRows, J.Ly) - 1, yn = y + 1 == J.Ly ? 0 : y + 1;
             const int trn = tr + 1 == J.trows ? 0 : tr + 1;
             const int tc = w / kTileWords, x0 = 32 * (w - tc * kTileWords);
             const uint32_t v = species_word(J, y, w), b = species_word(J, yn, w);
             const TileLabels A = tile_labels(J, s, tr * J.tcols + tc), B = tile_labels(J, s, trn * J.tcols + tc);
-            for (uint32_t m = straight_contacts(v, b); m != 0u; m &= m - 1u) {
+            for (uint32_t m = straight_contacts(v, b) & part; m != 0u; m &= m - 1u) {
                 const int p = __ffs(m) - 1;
                 unite(s.parent, A.bottom[x0 + run_start(v, p)], B.top[x0 + run_start(b, p)]);
             }
@@ -283,7 +292,7 @@ __global__ void cc_merge_kernel(const CcJob J, const ClusterScratch s, long long
             const bool left = w > 0 || !J.helical;
             const uint32_t vl = left ? (species_word(J, y, wl) >> end) & 1u : 0u;
             const uint32_t bw = left ? species_word(J, yn, wl) : 0u;
-            for (uint32_t m = slanted_contacts(v, b, (v << 1) | vl, (b << 1) | ((bw >> end) & 1u)); m != 0u;
+            for (uint32_t m = slanted_contacts(v, b, (v << 1) | vl, (b << 1) | ((bw >> end) & 1u)) & part; m != 0u;
                  m &= m - 1u) {
                 const int p = __ffs(m) - 1;
                 int32_t other;
@@ -296,7 +305,7 @@ __global__ void cc_merge_kernel(const CcJob J, const ClusterScratch s, long long
                 unite(s.parent, A.bottom[x0 + run_start(v, p)], other);
             }
         } else {
-            const long long k = it - (long long)J.trows * J.W;
+            const long long k = it - kParts * words;
             const int tc = (int)(k / J.Ly), y = (int)(k - (long long)tc * J.Ly);
             const bool wrap = tc + 1 == J.tcols;
             const int tcn = wrap ? 0 : tc + 1;
@@ -471,37 +480,41 @@ cc_count_kernel(const ClusterScratch s, int tiles, int slots, long long *sizes, 
 }
 
 // A lattice of at most 8 words by 1024 words in all, in one CTA: unions (with the
-// wraps), sizes, a histogram in the trees' memory and its compaction.
+// wraps), sizes, a histogram in the trees' memory and its compaction.  `parts` threads
+// (a power of two, at most 4) share a word, each with the contacts and the runs' starts in
+// its part: a word's unions wait for each other.  (64^2 with one / 4 / 8 threads: demixed
+// 19 / 12 / 12 us, columns of single sites 82 / 25 / 13, rows 6.7 / 6.5 / 8.5.)
 __global__ void __launch_bounds__(kSmallMaxThreads, 1)
-cc_small_kernel(const CcJob J, long long *sizes, long long *counts, long long capacity, long long *n_distinct)
+cc_small_kernel(const CcJob J, int parts, long long *sizes, long long *counts, long long capacity, long long *n_distinct)
 {
-    extern __shared__ __align__(16) int32_t parent[];  // a place per site of the words, then the counts
-    const int words = J.W * J.Ly, places = 32 * words;
-    const int stretched = places + words;  // entry e of the histogram is at e + e / 32
-    uint32_t *const cnt = (uint32_t *)(parent + stretched);
-    uint32_t *const bits = cnt + places / 2;
+    extern __shared__ __align__(16) int32_t parent[];  // the words' places, then the counts
+    const int words = J.W * J.Ly, places = kPlaces * words;  // entry e of the histogram is at e + e / 32
+    uint32_t *const cnt = (uint32_t *)(parent + places);
+    uint32_t *const bits = cnt + (places + 1) / 2;
     __shared__ int warp_tot[32];
     const int tid = threadIdx.x, T = blockDim.x;
-    const int y = tid / J.W, w = tid - y * J.W;
-    const bool in = tid < words;
+    const int word = tid / parts, y = word / J.W, w = word - y * J.W;
+    const bool in = word < words;
     const uint32_t v = in ? species_word(J, y, w) : 0u;
-    if (in) bits[tid] = v;
+    const int part0 = 32 / parts * (tid & (parts - 1));  // its first bit
+    const uint32_t part = (0xFFFFFFFFu >> (32 - 32 / parts)) << part0;
+    if (in && part0 == 0) bits[word] = v;
     for (int i = tid; i < places; i += T) parent[i] = i;
-    for (int i = tid; i < places / 2; i += T) cnt[i] = 0u;
+    for (int i = tid; i < (places + 1) / 2; i += T) cnt[i] = 0u;
     __syncthreads();
     if (in) {
         const int nlast = J.Lx - 32 * (J.W - 1);
         const int yn = y + 1 == J.Ly ? 0 : y + 1;
         const bool first = w == 0, lastw = w == J.W - 1;
         const int end = lastw ? nlast - 1 : 31;  // the word's last site
-        const int base = 32 * tid, below = 32 * (yn * J.W + w);
+        const int base = kPlaces * word, below = kPlaces * (yn * J.W + w);
         const uint32_t b = bits[yn * J.W + w];
         const int lw = first ? J.W - 1 : w - 1, lend = first ? nlast - 1 : 31;
         // the site to the right of the word's last one
         const int rw = lastw ? 0 : w + 1, ry = lastw && J.helical ? yn : y;
-        if (((v >> end) & 1u) && (bits[ry * J.W + rw] & 1u))
-            unite(parent, base + run_start(v, end), 32 * (ry * J.W + rw));
-        for (uint32_t m = straight_contacts(v, b); m != 0u; m &= m - 1u) {
+        if (((v & part) >> end & 1u) && (bits[ry * J.W + rw] & 1u))
+            unite(parent, base + run_start(v, end), kPlaces * (ry * J.W + rw));
+        for (uint32_t m = straight_contacts(v, b) & part; m != 0u; m &= m - 1u) {
             const int p = __ffs(m) - 1;
             unite(parent, base + run_start(v, p), below + run_start(b, p));
         }
@@ -513,29 +526,30 @@ cc_small_kernel(const CcJob J, long long *sizes, long long *counts, long long ca
             const uint32_t bl = (b << 1) | ((sl >> lend) & 1u);
             uint32_t m = slanted_contacts(v, b, (v << 1) | ((vl >> lend) & 1u), bl);
             if (carry) m = (m & ~1u) | (v & bl & 1u);  // its own bond: no straight contact stands for it
-            for (; m != 0u; m &= m - 1u) {
+            for (m &= part; m != 0u; m &= m - 1u) {
                 const int p = __ffs(m) - 1;
                 unite(parent, base + run_start(v, p),
-                      p > 0 ? below + run_start(b, p - 1) : 32 * (sy * J.W + lw) + run_start(sl, lend));
+                      p > 0 ? below + run_start(b, p - 1) : kPlaces * (sy * J.W + lw) + run_start(sl, lend));
             }
         }
     }
     __syncthreads();
-    for (uint32_t m = v & ~(v << 1); m != 0u; m &= m - 1u) {
+    const uint32_t starts = v & ~(v << 1) & part;
+    for (uint32_t m = starts; m != 0u; m &= m - 1u) {
         const int p = __ffs(m) - 1;
-        add_count(cnt, find_root((volatile int32_t *)parent, 32 * tid + p), (uint32_t)run_length(v, p), false);
+        add_count(cnt, find_root((volatile int32_t *)parent, kPlaces * word + p), (uint32_t)run_length(v, p), false);
     }
     __syncthreads();
-    for (int i = tid; i < stretched; i += T) parent[i] = 0;  // now the histogram: entry size - 1
+    for (int i = tid; i < places; i += T) parent[i] = 0;  // now the histogram: entry size - 1
     __syncthreads();
-    for (uint32_t m = v & ~(v << 1); m != 0u; m &= m - 1u) {
-        const uint32_t c = get_count(cnt, 32 * tid + __ffs(m) - 1);  // nonzero at roots only
+    for (uint32_t m = starts; m != 0u; m &= m - 1u) {
+        const uint32_t c = get_count(cnt, kPlaces * word + __ffs(m) - 1);  // nonzero at roots only
         if (c != 0u) atomicAdd(parent + (c - 1) + ((c - 1) >> 5), 1);
     }
     __syncthreads();
     // Compaction: every thread the entries of one contiguous part.
     const int lane = tid & 31, warp = tid >> 5, nw = T >> 5;
-    const int per = (places + T - 1) / T, e0 = min(tid * per, places), e1 = min(e0 + per, places);
+    const int sites = 32 * words, per = (sites + T - 1) / T, e0 = min(tid * per, sites), e1 = min(e0 + per, sites);
     int n = 0;
     for (int e = e0; e < e1; ++e) n += parent[e + (e >> 5)] != 0;
     int incl = n;
@@ -626,9 +640,11 @@ cudaError_t launch_cluster_histogram(const void *lat, int packing, int Lx, int L
     }
     if (e != cudaSuccess) return e;
     if (W <= kTileWords && (long long)W * Ly <= kSmallMaxThreads) {
-        const int words = W * Ly, threads = (words + 31) / 32 * 32;
-        cc_small_kernel<<<1, threads, (size_t)words * kSmallWordSmem, stream>>>(J, sizes, counts, capacity,
-                                                                                n_distinct);
+        int parts = 1;
+        while (parts < 4 && 2 * parts * W * Ly <= kSmallMaxThreads) parts *= 2;
+        const int words = W * Ly, threads = (parts * words + 31) / 32 * 32;
+        cc_small_kernel<<<1, threads, (size_t)words * kSmallWordSmem, stream>>>(J, parts, sizes, counts,
+                                                                                capacity, n_distinct);
         return cudaGetLastError();
     }
     J.tcols = (W + kTileWords - 1) / kTileWords;
@@ -637,7 +653,7 @@ cudaError_t launch_cluster_histogram(const void *lat, int packing, int Lx, int L
     const int tiles = J.tcols * J.trows;
     auto grid = [](long long n, long long most) { return (int)(n < 1 ? 1 : (n < most ? n : most)); };
     cc_tiles_kernel<<<grid(tiles, 152 * 4), kTileThreads, kTileSmem, stream>>>(J, s, tiles);
-    const long long items = (long long)J.trows * W + (long long)J.tcols * Ly;
+    const long long items = (long long)kParts * J.trows * W + (long long)J.tcols * Ly;
     cc_merge_kernel<<<grid((items + 127) / 128, 152 * 16), 128, 0, stream>>>(J, s, items);
     cc_sum_kernel<<<grid((tiles + 3) / 4, 152 * 16), 128, 0, stream>>>(s, tiles, J.slots);
     cc_count_kernel<<<grid((tiles + 15) / 16, 152 * 2), kCountThreads, 0, stream>>>(s, tiles, J.slots, sizes, counts,
