@@ -32,7 +32,7 @@ __device__ __forceinline__ uint32_t lattice_site(const void *lat, int packing, i
     return ((const uint8_t *)lat)[(size_t)y * pitch + x] ? 1u : 0u;
 }
 
-constexpr int kSnapRows = 8;  // image rows of a CTA
+constexpr int kSnapRows = 8;  // most image rows of a CTA
 
 // The column of a sample n of WS across, in half-sites: floor(u).  Site x of row y covers
 // half-sites 2x + y and 2x + y + 1, so the sample's site is (column - y) >> 1.
@@ -42,24 +42,24 @@ __device__ __forceinline__ int sample_column(long long n, long long U, long long
     return (int)((num | den) >> 32 ? num / den : (uint32_t)num / (uint32_t)den);
 }
 
-// A thread takes one image column of kSnapRows rows: its samples' columns are found once
+// A thread takes one image column of R <= kSnapRows rows: its samples' columns are found once
 // (a division each), the rows of the lattice that the CTA's image rows sample once per CTA.
 // Bound: a load, a shift and a few operations per sample.  ST: samples per pixel side, known
 // at compile time, or 0.  A 6143 x 3547 image of 8192^2 at 4 x 4 samples took 1158 us with two
 // 64-bit divisions per sample, 191 us so.
 template <int ST>
 __global__ void __launch_bounds__(kImgBlock)
-snapshot_kernel(const void *lat, int packing, int pitch, int Lx, int Ly, int W, int H, int S_, uint8_t *image,
+snapshot_kernel(const void *lat, int packing, int pitch, int Lx, int Ly, int W, int H, int S_, int R, uint8_t *image,
                 uint8_t *mask)
 {
     const int S = ST > 0 ? ST : S_;
     __shared__ int rows[kSnapRows * 64];
     const long long U = 2ll * Lx + Ly - 1;
-    const int strips = (H + kSnapRows - 1) / kSnapRows, cols = (W + kImgBlock - 1) / kImgBlock;
+    const int strips = (H + R - 1) / R, cols = (W + kImgBlock - 1) / kImgBlock;
     for (long long blk = blockIdx.x; blk < (long long)strips * cols; blk += gridDim.x) {
         const int strip = (int)(blk / cols);
         const int i = (int)(blk - (long long)strip * cols) * kImgBlock + (int)threadIdx.x;
-        const int j0 = strip * kSnapRows, nj = min(kSnapRows, H - j0);
+        const int j0 = strip * R, nj = min(R, H - j0);
         __syncthreads();
         for (int k = threadIdx.x; k < nj * S; k += kImgBlock)
             rows[k] = sample_column((long long)j0 * S + k, Ly, (long long)H * S);  // floor(v) likewise
@@ -206,12 +206,17 @@ int img_grid(long long work)
 cudaError_t launch_snapshot(const void *lat, int packing, int pitch, int Lx, int Ly, int W, int H, int S,
                             uint8_t *image, uint8_t *mask, cudaStream_t stream)
 {
-    const long long strips = (H + kSnapRows - 1) / kSnapRows, cols = (W + kImgBlock - 1) / kImgBlock;
+    // Small images take fewer rows per CTA, so that the chip is in use: 64 x 64 at 7 x 7 samples of
+    // 8192^2 37 us with 8 rows, 8.6 with one; 300 x 300 at 5 x 5 of 300^2 19 and 8.7.
+    const long long cols = (W + kImgBlock - 1) / kImgBlock;
+    int R = kSnapRows;
+    while (R > 1 && (H + R - 1) / R * cols < 152 * 4) R /= 2;
+    const long long strips = (H + R - 1) / R;
     const int g = (int)(strips * cols < 152 * 64 ? strips * cols : 152 * 64);
     auto kernel = S == 1 ? snapshot_kernel<1>
                 : (S == 2 ? snapshot_kernel<2> : (S == 3 ? snapshot_kernel<3> : (S == 4 ? snapshot_kernel<4>
                                                                                            : snapshot_kernel<0>)));
-    kernel<<<g, kImgBlock, 0, stream>>>(lat, packing, pitch, Lx, Ly, W, H, S, image, mask);
+    kernel<<<g, kImgBlock, 0, stream>>>(lat, packing, pitch, Lx, Ly, W, H, S, R, image, mask);
     return cudaGetLastError();
 }
 
