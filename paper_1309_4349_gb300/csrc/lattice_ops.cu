@@ -364,11 +364,20 @@ __global__ void ffn_kernel(const void *lat, int packing, int Lx, int Ly, int pit
                 e2 = __funnelshift_r(e2, k >> 2, 1);
             }
         };
+        // the groups of four that hold the word's sites: 8, or 9, fewer in a row's last word
+        // (4 x 200000: 12.8 us with 8 for every word, 8.0 so)
+        const uint32_t groups = (off + (uint32_t)min(32, Lx - 32 * w) + 3u) >> 2;
+        const uint32_t first8 = min(groups, 8u);
 #pragma unroll 2
-        for (int g = 0; g < 8; ++g) push((site >> 2) + (uint32_t)g, d0, d1, d2);
+        for (uint32_t g = 0; g < first8; ++g) push((site >> 2) + g, d0, d1, d2);
+        if (first8 < 8u) {
+            d0 >>= 32u - 4u * first8;
+            d1 >>= 32u - 4u * first8;
+            d2 >>= 32u - 4u * first8;
+        }
         if (off != 0u) {
             uint32_t h0 = 0u, h1 = 0u, h2 = 0u;  // four more, in the top bits
-            push((site >> 2) + 8u, h0, h1, h2);
+            if (groups > 8u) push((site >> 2) + 8u, h0, h1, h2);
             d0 = __funnelshift_r(d0, h0 >> 28, off);
             d1 = __funnelshift_r(d1, h1 >> 28, off);
             d2 = __funnelshift_r(d2, h2 >> 28, off);
