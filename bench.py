@@ -78,11 +78,11 @@ ISSUE_LANES_PER_SM = 128
 # 4-phase band launch of the 8192x8192 lattice; one resident helical launch of 500
 # MCS of one 402x399 lattice), valid only for the kernel sources they were taken
 # with (hash of the kernel's file + sweep_common.cuh + cluster_exchange.cuh + philox.cuh).
-TRAFFIC_C2_LAUNCH = 230656
+TRAFFIC_C2_LAUNCH = 228352
 TRAFFIC_C3_LAUNCH = 8494336
-TRAFFIC_SOURCES = "650cc4995f465648"
-TRAFFIC_C6_LAUNCH = 93184
-TRAFFIC_HELICAL_SOURCES = "56a8f01e6f3bbf26"
+TRAFFIC_SOURCES = "1f49b93f7c6e3a4b"
+TRAFFIC_C6_LAUNCH = 91648
+TRAFFIC_HELICAL_SOURCES = "2cd06f1b9a4cacfc"
 
 # Kernels launched per library call (fixed by the library's structure).
 LAUNCHES_SWEEP = 1

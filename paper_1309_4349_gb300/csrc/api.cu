@@ -177,8 +177,8 @@ int cluster_for_rows(int Lx, int Ly, int min_rows)
 }
 
 // Automatic cluster size: bands of at least 16 rows.  More CTAs shorten each phase
-// (GB300, us per phase with half as many CTAs and with these: 64^2 0.82 / 0.76, 128^2
-// 0.93 / 0.85, 256^2 1.06 / 0.96, 300^2 1.18 / 1.04).
+// (GB300, us per phase with half as many CTAs and with these: 64^2 0.77 / 0.70, 128^2
+// 0.87 / 0.79, 256^2 1.00 / 0.89, 300^2 1.09 / 0.94).
 constexpr int kLatencyRows = 16;
 int auto_cluster(int Lx, int Ly) { return cluster_for_rows(Lx, Ly, kLatencyRows); }
 
@@ -254,8 +254,8 @@ constexpr int kThroughputRows = 64;
 
 // Lattices of at least this many sites run faster on the tiled path, whose bands
 // use every SM, than in one cluster's shared memory (GB300, 200 MCS of square TRI6
-// lattices: 724^2 5.7 vs 4.8 ms resident, 1024^2 5.8 vs 7.1 ms, 2048^2 6.8 vs
-// 20.1 ms); the automatic shape of a standalone handle takes it there.
+// lattices: 724^2 5.0 vs 3.1 ms resident, 900^2 4.4 vs 4.2, 1024^2 4.4 vs 4.9, 2048^2
+// 6.0 vs 15.3); the automatic shape of a standalone handle takes it there.
 constexpr long long kTiledAutoSites = 786432;
 
 // standalone: a handle of its own (klmc_create, klmc_create_ex), which may take the
@@ -324,7 +324,9 @@ klmc_status create_one(klmc_ctx **out, const klmc_params *p, klmc_batch *owner, 
     J.packing = c->p.packing;
     J.geometry = p->geometry;
     J.W = c->W;
-    J.RW = (p->Lx + 95) / 32;  // ceil(Lx / 32) + 2: windows read words j .. j+2
+    // A shared-memory row's stride, two words more than its sites fill: what fits a cluster, and
+    // with it the shapes and plans that handles report, is counted so.
+    J.RW = (p->Lx + 95) / 32;
     J.magicW = (0x100000000ull + (unsigned long long)c->W - 1) / (unsigned long long)c->W;
     J.key0 = (uint32_t)p->seed;
     J.key1 = (uint32_t)(p->seed >> 32);

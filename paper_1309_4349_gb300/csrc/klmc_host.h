@@ -73,7 +73,9 @@ void destroy(klmc_ctx *c);
 size_t device_bytes(const klmc_params *p);
 
 // Model of one step's time (8 phases) of the resident kernel at a launch shape:
-// 1.3 us per phase plus 1 us per round of anchor words per thread.
+// 1.3 us per phase plus 1 us per round of anchor words per thread.  It was fitted to
+// earlier kernels: a phase of 64^2 on 4 CTAs of 256 threads takes 0.70 us where it says
+// 2.3, of 400^2 on 16 of 512 1.09 (2.3), of 400^2 on 2 of 128 5.5 (12.3).
 inline double model_mcs_us(int Lx, int Ly, int cluster, int threads)
 {
     const double words = (double)((Lx + 31) / 32);

@@ -87,10 +87,11 @@ namespace {
 
 double seconds(const klmc_server *s) { return std::chrono::duration<double>(Clock::now() - s->t0).count(); }
 
-// Steps per round: about 4 ms of work for every job at the launch shape it runs
-// with this round.
 constexpr int kHelicalStreams = 8;  // streams for the helical jobs of a round
 
+// Steps per round: 4 ms of every job's work by the time model, at the launch shape it runs
+// with this round.  The kernels take 0.3 to 0.5 of what the model says, so that a round
+// lasts 1.2 to 1.9 ms.
 int64_t quantum(const Job *j, std::pair<int, int> shape)
 {
     const klmc_ctx *c = j->ctx;

@@ -27,7 +27,7 @@
 // sweep boundaries (seven per sweep).  A thread's first word is the same in every
 // iteration, so its place and ends are found once; the next iteration's schedule entry
 // and draw key are prepared by one lane.  Bound: the instructions of an iteration's
-// busiest warp (402 x 399 on 16 CTAs: 1.26 us per iteration; 1.88 with copies of the row
+// busiest warp (402 x 399 on 16 CTAs: 1.24 us per iteration; 1.88 with copies of the row
 // ends and a cluster barrier per exchange).
 #include <string.h>
 

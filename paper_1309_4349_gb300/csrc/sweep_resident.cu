@@ -988,9 +988,9 @@ band_phases_kernel(const SweepJob J, const void *__restrict__ src, void *__restr
     if (bulk && tid < 32) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
-// Three variants: 512 threads (one CTA per SM; single lattices on one CTA), 256
-// threads with at most 128 registers (two CTAs per SM) and 128 threads with at
-// most 128 registers (four CTAs per SM; batches of many lattices).
+// Three variants: 512 threads (one CTA per SM; phases of many words), 256 threads with
+// at most 128 registers (two CTAs per SM), of both the last warp without tasks, and 128
+// threads with at most 128 registers (four CTAs per SM; batches of many lattices).
 template <int THREADS, int MINB>
 cudaError_t configure_once()
 {
@@ -1072,9 +1072,9 @@ int resident_block_phases(int Lx, int Ly, int cluster) { return block_phases(Lx,
 
 // A phase of a lattice spread over a cluster lasts as long as its busiest warp, so the
 // CTA has enough threads for one task each: 224 of 256 or 480 of 512 run tasks (the
-// others prepare).  GB300, us per phase at 256 / 512 threads: 64^2 on 2 CTAs 0.79 /
-// 0.83, 280^2 on 16 0.94 / 0.96, 330^2 on 16 (198 words a phase) 1.04 / 1.04, 262^2 on
-// 8 (216) 1.04 / 1.07, 400^2 on 16 (260) 1.41 / 1.12.
+// others prepare).  GB300, us per phase at 256 / 512 threads: 64^2 on 2 CTAs 0.77 /
+// 0.80, 280^2 on 16 0.91 / 0.93, 330^2 on 16 (198 words a phase) 1.01 / 1.01, 262^2 on
+// 8 (216) 1.01 / 1.04, 400^2 on 16 (260) 1.21 / 1.09.
 int resident_default_threads(int Lx, int Ly, int cluster)
 {
     const int C = cluster < 1 ? 1 : cluster, K = block_phases(Lx, Ly, C);
