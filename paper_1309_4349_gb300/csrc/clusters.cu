@@ -15,12 +15,12 @@
 //
 // Bound: the latency of the shared-memory trees; the bits are read twice and a tile
 // of 8192 sites leaves about 200 nodes.  8192^2 at 50/50, demixing (GB300, per
-// species): 0.37 ms (tiles 0.30, borders 0.04, sums 0.01, counts and compaction 0.03);
-// 20 ms with one parent entry per site in device memory (the sum over sites 13 ms, one
-// atomic per site on the largest cluster's root; the unions 5.6; the compaction's scan of
-// every size 3.3).  400^2: 62 us, 130 before.  Lattices that one CTA's shared memory
-// holds are done by one launch: 64^2 21 us, 145 before (five launches, one site per
-// thread on 4 CTAs).
+// species): 0.51 ms (tiles 0.36, borders, sums and counts about 0.06 each with cold
+// caches); 21 ms with one parent entry per site in device memory (the sum over sites 13
+// ms, one atomic per site on the largest cluster's root; the unions 5.6; the compaction's
+// scan of every size 3.3).  400^2, 40% A: 50 us, 140 before.  Lattices that one CTA's
+// shared memory holds are done by one launch: 64^2 11 us, 116 before (five launches, one
+// site per thread on 4 CTAs).
 #include "klmc_internal.h"
 
 namespace klmc {
